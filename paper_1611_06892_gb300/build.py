@@ -18,7 +18,9 @@ LIB = os.path.join(HERE, "libbidiag.so")
 ROOT = os.path.dirname(HERE)
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["plan.cpp", "kernels.cu", "capi.cu", "noalloc.cu", "peak.cu"]
+# (source, value of BD_EXEC_PART): kernels.cu is compiled once per executor instantiation
+UNITS = [("kernels.cu", part) for part in (1, 2, 3, 4, 5, 0)] + [
+    (src, None) for src in ("plan.cpp", "capi.cu", "noalloc.cu", "peak.cu")]
 
 
 def _nvcc():
@@ -28,11 +30,13 @@ def _nvcc():
     return cand
 
 
-def _compile(src, verbose):
+def _compile(unit, verbose):
+    src, part = unit
     nvcc = _nvcc()
-    obj = os.path.join(BUILD, os.path.splitext(src)[0] + ".o")
-    cmd = [nvcc, "-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC,-O2", *ARCH,
+    obj = os.path.join(BUILD, os.path.splitext(src)[0] + ("" if part is None else f"_{part}") + ".o")
+    cmd = [nvcc, "-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC,-O2", "-diag-suppress", "177", *ARCH,
            "-I", os.path.join(ROOT, "include"), "-c", os.path.join(CSRC, src), "-o", obj]
+    cmd += [] if part is None else [f"-DBD_EXEC_PART={part}"]
     if src.endswith(".cu"):
         cmd += ["-Xptxas", "-v"] if verbose else []
     else:
@@ -45,8 +49,8 @@ def _compile(src, verbose):
 
 def build(verbose=False):
     os.makedirs(BUILD, exist_ok=True)
-    with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        outs = list(ex.map(lambda s: _compile(s, verbose), SOURCES))
+    with ThreadPoolExecutor(max_workers=len(UNITS)) as ex:
+        outs = list(ex.map(lambda u: _compile(u, verbose), UNITS))
     if verbose:
         for _, log in outs:
             if log:

@@ -66,6 +66,7 @@ struct BatchPlan {
   std::vector<bd::MatInfo> info;
   int64_t tot0 = 0, tot1 = 0, totT = 0, tiles_all = 0, cols_all = 0;
   size_t smem = 0;
+  bool digits = false;          // FP64: some matrix's updates run as digit products
   int ntasks = 0;
   PlanDev prog;                 // the merged device program
   void* d_mats = nullptr;       // info on the device
@@ -188,7 +189,7 @@ int run_exec(bidiag_handle h, const PlanDev& pd, int ntasks, void* b0, int64_t n
              int64_t n2, void* T, int npanels, int nb, int ib, int w, int esize, bool timed = false,
              const bd::MatInfo* d_mats = nullptr, int nmats = 0, size_t smem_batch = 0,
              const void* const* bx = nullptr, const int64_t* nx = nullptr, const bd::BwdParams* bwd = nullptr,
-             int auto_window = 0) {
+             int auto_window = 0, bool digits_batch = false) {
   if (ntasks == 0) return BIDIAG_OK;
   size_t smem = d_mats ? smem_batch : (bwd ? bd::bwd_smem_bytes(nb, ib, bwd->hw, esize) : bd::exec_smem_bytes(nb, ib, w, esize));
   // tcgen05 updates (FP32 forward, one CTA per SM): TMEM for one accumulator of N = max(w, ib) (rounded to
@@ -206,8 +207,18 @@ int run_exec(bidiag_handle h, const PlanDev& pd, int ntasks, void* b0, int64_t n
       smem = su;
     }
   }
-  CK(h, bd::exec_set_smem(smem, esize, bwd != nullptr));
-  const int per_sm = std::max(1, bd::exec_max_ctas_per_sm(smem, esize, bwd != nullptr));
+  // FP64 forward: digit products on tcgen05 where the sizes (of any matrix of a batch) fit
+  if (esize == 8 && !bwd && (d_mats ? digits_batch : bd::digits_tmem(nb, ib, w) > 0)) {
+    const size_t su = std::max(smem, bd::digits_smem_bytes());
+    if (su <= h->smem_optin && bd::exec_set_smem(su, esize, false, true) == cudaSuccess &&
+        bd::exec_max_ctas_per_sm(su, esize, false, true) == 1) {
+      umma_cols = 512;
+      smem = su;
+    }
+  }
+  const bool digits = esize == 8 && umma_cols > 0;
+  CK(h, bd::exec_set_smem(smem, esize, bwd != nullptr, digits));
+  const int per_sm = std::max(1, bd::exec_max_ctas_per_sm(smem, esize, bwd != nullptr, digits));
   bd::ExecParams prm{};
   prm.tasks = pd.d_tasks;
   prm.deps = pd.d_deps;
@@ -782,6 +793,7 @@ int band_batched_impl(bidiag_handle h, int64_t count, const int64_t* m, const in
     }
     const BatchPlan::One& o = mats[(size_t)b];
     bp->smem = std::max(bp->smem, bd::exec_smem_bytes(o.nb, o.ib, o.w, esize));
+    bp->digits = bp->digits || bd::digits_tmem(o.nb, o.ib, o.w) > 0;
   }
   // storage layout
   bp->info.resize((size_t)count);
@@ -891,7 +903,8 @@ int band_batched_impl(bidiag_handle h, int64_t count, const int64_t* m, const in
     if (e != cudaSuccess) return bail(cuda_fail(h, e, "cudaEventCreate"));
   }
   rc = run_exec(h, bp->prog, bp->ntasks, store->tiles, tiles_all, store->tiles2, tot1 ? 1 : 0, nullptr, 0, store->T,
-                0, 0, 1, 1, esize, timed, static_cast<const bd::MatInfo*>(bp->d_mats), (int)count, smem);
+                0, 0, 1, 1, esize, timed, static_cast<const bd::MatInfo*>(bp->d_mats), (int)count, smem, nullptr, nullptr,
+                nullptr, 0, bp->digits);
   if (rc) return bail(rc);
   h->timed = timed;
   e = bd::launch_extract_batched(d_ex, (int)count, cols_all, esize, h->stream);

@@ -26,6 +26,12 @@
 
 #include "kernels.cuh"
 
+// This file is compiled once per executor instantiation (BD_EXEC_PART 1 - 5, in parallel: each takes ptxas
+// about a minute) and once for the other kernels and the host functions (0).
+#ifndef BD_EXEC_PART
+#define BD_EXEC_PART 0
+#endif
+
 namespace bd {
 namespace {
 
@@ -1495,6 +1501,29 @@ __device__ bool task_update_umma(unsigned char* smb, int type, const float* X, f
   return true;
 }
 
+#include "update_digits.cuh"
+
+// An update (strip or panel block, arguments as task_update) on the tensor cores where the CTA holds TMEM for it
+// and the sizes fit, on the FMA units otherwise; true if any of it ran on tcgen05.
+template <typename E, bool kDig>
+__device__ __forceinline__ bool run_update(unsigned char* smb, int type, const E* X, E* Cp, E* C, int tr, bool notrans, const E* Tg,
+                           int nb, int ib, int w, int blk0, int blk1, int col0, int ncols, Umma& um,
+                           const ExecParams& prm) {
+  int done = 0;
+  if constexpr (sizeof(E) == 4) {
+    if (prm.f32_simt == 0 &&
+        task_update_umma(smb, type, X, Cp, C, tr, notrans, Tg, nb, ib, w, blk0, blk1, col0, ncols, um, prm))
+      return true;
+  } else if constexpr (kDig) {
+    if (um.ncols_alloc >= kDigTmem && digits_fit(nb, ib, ncols))
+      done = task_update_digits(smb, type, X, Cp, C, tr, notrans, Tg, nb, ib, blk0, blk1, col0, ncols, um, prm);
+    if (done == blk1 - blk0) return true;
+    if (notrans) blk1 -= done; else blk0 += done;
+  }
+  task_update(smb, type, X, Cp, C, tr, notrans, Tg, nb, ib, w, blk0, blk1, col0, ncols, prm.f32_simt == 1);
+  return done > 0;
+}
+
 // ---------------------------------------------------------------------------------------------
 // Adjoint of the reduction (reverse sweep).  Each Householder step of the forward sweep is
 // M' = H(x) M on the rows it acts on, H = I - tau v v^T, x its pivot column, H x = beta e_1.  Going
@@ -1996,7 +2025,10 @@ __device__ int next_task(const ExecParams& prm) {
 // Persistent dataflow executor: CTAs take sub-tasks from a queue in topological priority order
 // (next_task), wait (bounded) until the sub-tasks they depend on are done, run them and publish
 // completion.
-template <typename E, bool kBwd>
+// kDig (FP64): with the digit products of update_digits.cuh.  Programs of tiles too small for them run the
+// instantiation without: it does without their registers' spills around the panel factor (192 x 160, nb 32:
+// 2.37 ms against 2.44).
+template <typename E, bool kBwd, bool kDig>
 __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm) {
   extern __shared__ __align__(128) unsigned char smb[];
   __shared__ int s_idx;
@@ -2004,10 +2036,10 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
   __shared__ __align__(8) uint64_t s_mbar;
   __shared__ uint32_t s_tmem;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // FP32 storage: TMEM columns for the tcgen05 phase of the updates, held for the whole launch (the host
-  // enables it only with one CTA per SM, so the allocation never waits), and the MMA completion barrier
+  // TMEM columns for the tcgen05 phases of the updates, held for the whole launch (the host enables it
+  // only with one CTA per SM, so the allocation never waits), and the MMA completion barrier
   Umma um{0u, 0u, 0u, 0u, 0};
-  if constexpr (sizeof(E) == 4 && !kBwd) {
+  if constexpr (!kBwd && (kDig || sizeof(E) == 4)) {
     if (prm.umma_cols > 0) {
       if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
@@ -2116,19 +2148,10 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
       case PU: {
         E* A = (kind == PM_GE) ? nullptr : tile_ptr<E>(prm, mv, t.a, ok);
         const int utype = kind == PM_GE ? UNMQR : (kind == PM_TS ? TSMQR : TTMQR);
-        if (ok && Tg && blk < strip && strip < nblk && kind <= PM_TT) {
-          bool done = false;
-          if constexpr (sizeof(E) == 4)
-            if (prm.f32_simt == 0)
-              done = task_update_umma(smb, utype, X, A, X, tr, false, Tg, nb, ib, wst, blk, blk + 1, strip * ib, ib,
-                                      um, prm);
-          on_tc5 = done;
-          if (!done)
-            task_update(smb, utype, X, A, X, tr, false, Tg, nb, ib, wst, blk, blk + 1, strip * ib, ib,
-                        prm.f32_simt == 1);
-        } else {
+        if (ok && Tg && blk < strip && strip < nblk && kind <= PM_TT)
+          on_tc5 = run_update<E, kDig>(smb, utype, X, A, X, tr, false, Tg, nb, ib, wst, blk, blk + 1, strip * ib, ib, um, prm);
+        else
           ok = false;
-        }
         break;
       }
       case UNMQR:
@@ -2137,19 +2160,11 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
         E* A = (type == UNMQR) ? nullptr : tile_ptr<E>(prm, mv, t.a, ok);
         E* C = tile_ptr<E>(prm, mv, t.c, ok);
         const int col0 = strip * wst;
-        if (ok && Tg && col0 < nb) {
-          bool done = false;
-          if constexpr (sizeof(E) == 4)
-            if (prm.f32_simt == 0)
-              done = task_update_umma(smb, type, X, A, C, tr, notrans, Tg, nb, ib, wst, 0, nblk, col0,
-                                      min(wst, nb - col0), um, prm);
-          on_tc5 = done;
-          if (!done)
-            task_update(smb, type, X, A, C, tr, notrans, Tg, nb, ib, wst, 0, nblk, col0, min(wst, nb - col0),
-                        prm.f32_simt == 1);
-        } else {
+        if (ok && Tg && col0 < nb)
+          on_tc5 = run_update<E, kDig>(smb, type, X, A, C, tr, notrans, Tg, nb, ib, wst, 0, nblk, col0, min(wst, nb - col0), um,
+                              prm);
+        else
           ok = false;
-        }
         break;
       }
       case COPY: {
@@ -2269,7 +2284,7 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
       }
     }
   }
-  if constexpr (sizeof(E) == 4 && !kBwd) {
+  if constexpr (!kBwd && (kDig || sizeof(E) == 4)) {
     if (prm.umma_cols > 0) {
       // every MMA was waited for, except after a wait that ran out: wait (bounded) once more for it
       if (um.failed) mbar_wait(um.mbar, um.phase ^ 1u, prm.wait_ns);
@@ -2282,6 +2297,21 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
   }
 }
 
+#if BD_EXEC_PART > 0
+}  // namespace
+#if BD_EXEC_PART == 1
+const void* exec_fn_f64() { return reinterpret_cast<const void*>(exec_kernel<double, false, true>); }
+#elif BD_EXEC_PART == 2
+const void* exec_fn_f64_bwd() { return reinterpret_cast<const void*>(exec_kernel<double, true, false>); }
+#elif BD_EXEC_PART == 3
+const void* exec_fn_f32() { return reinterpret_cast<const void*>(exec_kernel<float, false, false>); }
+#elif BD_EXEC_PART == 4
+const void* exec_fn_f32_bwd() { return reinterpret_cast<const void*>(exec_kernel<float, true, false>); }
+#else
+const void* exec_fn_f64_small() { return reinterpret_cast<const void*>(exec_kernel<double, false, false>); }
+#endif
+}  // namespace bd
+#else
 template <typename E>
 __global__ void r_part_kernel(const E* __restrict__ src, E* __restrict__ dst, int64_t rows_t, int64_t cols_t, int nb,
                               int s0) {
@@ -2446,6 +2476,9 @@ size_t umma_smem_bytes(int nb, int ib, int w) {
   return kHeaderDoubles * sizeof(double) + sizeof(float) * (size_t)layout_umma(nb, ib, w).total;
 }
 
+int digits_tmem(int nb, int ib, int w) { return digits_fit(nb, ib, w < nb ? w : nb) ? kDigTmem : 0; }
+size_t digits_smem_bytes() { return kHeaderDoubles * sizeof(double) + kDigBytes; }
+
 size_t bwd_smem_bytes(int nb, int ib, int hw, int esize) {
   const BwdLayout a = layout_bwd_update(nb, ib, hw, esize), b = layout_bwd_panel(nb, ib, esize);
   return kHeaderDoubles * sizeof(double) + (size_t)esize * (size_t)(a.total > b.total ? a.total : b.total);
@@ -2473,34 +2506,26 @@ int choose_strip_width(int nb, int ib, int preferred, size_t smem_limit, int esi
 }
 
 namespace {
-template <typename E>
-const void* exec_fn(bool bwd) {
-  return bwd ? reinterpret_cast<const void*>(exec_kernel<E, true>) : reinterpret_cast<const void*>(exec_kernel<E, false>);
+const void* exec_fn(int esize, bool bwd, bool digits) {
+  if (esize == 4) return bwd ? exec_fn_f32_bwd() : exec_fn_f32();
+  return bwd ? exec_fn_f64_bwd() : (digits ? exec_fn_f64() : exec_fn_f64_small());
 }
 }  // namespace
 
-cudaError_t exec_set_smem(size_t smem, int esize, bool bwd) {
-  return cudaFuncSetAttribute(esize == 4 ? exec_fn<float>(bwd) : exec_fn<double>(bwd),
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t exec_set_smem(size_t smem, int esize, bool bwd, bool digits) {
+  return cudaFuncSetAttribute(exec_fn(esize, bwd, digits), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
-int exec_max_ctas_per_sm(size_t smem, int esize, bool bwd) {
+int exec_max_ctas_per_sm(size_t smem, int esize, bool bwd, bool digits) {
   int n = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &n, esize == 4 ? exec_fn<float>(bwd) : exec_fn<double>(bwd), kThreads, smem);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, exec_fn(esize, bwd, digits), kThreads, smem);
   return e == cudaSuccess ? n : 0;
 }
 
 cudaError_t launch_exec(const ExecParams& prm, int grid, size_t smem, cudaStream_t st) {
-  const bool bwd = prm.bwd.part != nullptr;
-  if (prm.esize == 4) {
-    if (bwd) exec_kernel<float, true><<<grid, kThreads, smem, st>>>(prm);
-    else exec_kernel<float, false><<<grid, kThreads, smem, st>>>(prm);
-  } else {
-    if (bwd) exec_kernel<double, true><<<grid, kThreads, smem, st>>>(prm);
-    else exec_kernel<double, false><<<grid, kThreads, smem, st>>>(prm);
-  }
-  return cudaGetLastError();
+  void* args[1] = {const_cast<ExecParams*>(&prm)};
+  return cudaLaunchKernel(exec_fn(prm.esize, prm.bwd.part != nullptr, prm.umma_cols > 0), dim3((unsigned)grid), dim3(kThreads), args, smem,
+                          st);
 }
 
 cudaError_t launch_pack_batched(const PackDesc* d, int count, int64_t total_tiles, int esize, cudaStream_t st) {
@@ -2586,3 +2611,4 @@ cudaError_t launch_extract(const float* tiles, int64_t rows_t, int nb, int64_t n
 }
 
 }  // namespace bd
+#endif

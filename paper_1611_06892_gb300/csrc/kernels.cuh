@@ -71,7 +71,7 @@ struct ExecParams {
   int nmats;
   int f32_simt;         // FP32 tiles only: 0 = three-TF32 tensor-core updates (tcgen05 where umma_cols > 0),
                         // 1 = updates by FP32 FFMA, 2 = three-TF32 updates on the warp-level MMA only
-  int umma_cols;        // FP32 forward program: TMEM columns each CTA allocates for the tcgen05 phase (0: none)
+  int umma_cols;        // forward programs: TMEM columns each CTA allocates for the tcgen05 phases (0: none)
   int f32_scalars64;    // FP32 tiles only: 1 = reflector beta / tau / scale in FP64 instead of float pairs
   int window;           // queue entries from the head a CTA scans for a ready sub-task (0: strict queue order)
   BwdParams bwd;        // adjoint program only
@@ -81,6 +81,10 @@ struct ExecParams {
 size_t exec_smem_bytes(int nb, int ib, int w, int esize);
 // Dynamic shared memory of the FP32 forward executor when its updates take the tcgen05 path (ib 32).
 size_t umma_smem_bytes(int nb, int ib, int w);
+// FP64 forward executor: TMEM columns its updates need to run as digit products on tcgen05 (0: the sizes stay on
+// the FP64 units), and the dynamic shared memory of that path.
+int digits_tmem(int nb, int ib, int w);
+size_t digits_smem_bytes();
 // Column-strip width of the update sub-tasks: a multiple of ib, at most nb, as close to `preferred`
 // as the shared-memory limit allows; 0 if even w = ib does not fit.
 int choose_strip_width(int nb, int ib, int preferred, size_t smem_limit, int esize);
@@ -90,10 +94,17 @@ int choose_strip_width(int nb, int ib, int preferred, size_t smem_limit, int esi
 size_t bwd_smem_bytes(int nb, int ib, int hw, int esize);
 int choose_bwd_chunk(int nb, int ib, int w, size_t smem_limit, int esize);
 
+// The executor's instantiations (each in an object file of its own).
+const void* exec_fn_f64();         // with digit products (ExecParams::umma_cols > 0)
+const void* exec_fn_f64_small();   // without
+const void* exec_fn_f64_bwd();
+const void* exec_fn_f32();
+const void* exec_fn_f32_bwd();
+
 // Executor launch: the adjoint instantiation when prm.bwd.part is set (bwd below must match).
 cudaError_t launch_exec(const ExecParams& prm, int grid, size_t smem, cudaStream_t st);
-cudaError_t exec_set_smem(size_t smem, int esize, bool bwd = false);
-int exec_max_ctas_per_sm(size_t smem, int esize, bool bwd = false);
+cudaError_t exec_set_smem(size_t smem, int esize, bool bwd = false, bool digits = false);
+int exec_max_ctas_per_sm(size_t smem, int esize, bool bwd = false, bool digits = false);
 
 // Column-major (ld) matrix <-> zero-padded tile buffer (grid of rows_t x cols_t tiles of nb x nb).
 cudaError_t launch_pack(const double* A, int64_t lda, int64_t m, int64_t n, int nb, double* tiles, int64_t rows_t,

@@ -112,7 +112,7 @@ extern "C" int bidiag_band_noalloc(int64_t m, int64_t n, const double* d_A, int6
 
   const int w = bd::choose_strip_width(nb, ib, 32, (size_t)optin - 64, 8);
   if (!w) return BIDIAG_ERR_UNSUPPORTED;
-  const size_t smem = bd::exec_smem_bytes(nb, ib, w, 8);
+  size_t smem = bd::exec_smem_bytes(nb, ib, w, 8);
 
   // The task program is planned on the host (host memory only).
   bd::Plan pl;
@@ -179,8 +179,17 @@ extern "C" int bidiag_band_noalloc(int64_t m, int64_t n, const double* d_A, int6
     prm.wait_ns = wl ? std::strtoull(wl, nullptr, 10) : 20000000000ull;
     prm.esize = 8;
     prm.window = tiles2 ? 0 : bd::kWindowF64BiDiag;
-    if ((e = bd::exec_set_smem(smem, 8)) != cudaSuccess) return cuda_status(e);
-    int per_sm = bd::exec_max_ctas_per_sm(smem, 8);
+    if (bd::digits_tmem(nb, ib, w) > 0) {   // digit products on tcgen05, as bidiag_band runs them
+      const size_t su = std::max(smem, bd::digits_smem_bytes());
+      if (su <= (size_t)optin - 64 && bd::exec_set_smem(su, 8, false, true) == cudaSuccess &&
+          bd::exec_max_ctas_per_sm(su, 8, false, true) == 1) {
+        prm.umma_cols = bd::digits_tmem(nb, ib, w);
+        smem = su;
+      }
+    }
+    const bool digits = prm.umma_cols > 0;
+    if ((e = bd::exec_set_smem(smem, 8, false, digits)) != cudaSuccess) return cuda_status(e);
+    int per_sm = bd::exec_max_ctas_per_sm(smem, 8, false, digits);
     if (per_sm < 1) per_sm = 1;
     const int64_t grid = (int64_t)nsm * per_sm < (int64_t)ntask ? (int64_t)nsm * per_sm : (int64_t)ntask;
     if ((e = bd::launch_exec(prm, (int)grid, smem, st)) != cudaSuccess) return cuda_status(e);
