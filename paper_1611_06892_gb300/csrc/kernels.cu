@@ -22,21 +22,22 @@
 // Householder convention (LAPACK style): for x = [alpha; tail], sigma2 = tail . tail; sigma2 == 0 gives
 // H = I (tau = 0, beta = alpha); otherwise beta = -sgn(alpha) sqrt(alpha^2 + sigma2) with sgn(alpha) = -1
 // only for alpha < 0, tau = (beta - alpha) / beta, v = [1; tail / (alpha - beta)].
-#include <cstdio>
-
-#include "kernels.cuh"
-
 // This file is compiled once per executor instantiation (BD_EXEC_PART 1 - 5, in parallel: each takes ptxas
 // about a minute) and once for the other kernels and the host functions (0).
 #ifndef BD_EXEC_PART
 #define BD_EXEC_PART 0
 #endif
+#include <cstdio>
+
+#include "kernels.cuh"
+
 
 namespace bd {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWarps = kThreads / 32;
+constexpr int kSmemAlign = BD_EXEC_PART == 1 ? 1024 : 128;   // (swizzled MMA operands)
 
 template <typename E> struct Vec2;
 template <> struct Vec2<double> { using type = double2; };
@@ -203,39 +204,40 @@ __device__ __forceinline__ void put(E* s, E* hi, int i, E v) {
   s[i] = v;
 }
 
-// Up to 256 x 32 elements: all of a thread's loads (up to 32) are issued before the first shared store, so
+// Up to 256 x 32 elements: all of a thread's loads (up to 32, with 512 threads 16) are issued before the first shared store, so
 // that one L2 latency covers the whole block.  Lanes run along the contiguous direction of global memory.
 template <typename E>
 __device__ __forceinline__ void load_block32(E* s, int rs, int cs, const E* g, int nb, int tr, int r0, int c0,
                                              int rows, int cols, int mask, E* hi) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  E v[32];
-  if (!tr) {   // c = warp + 8 kc, r = lane + 32 kr
+  constexpr int kN = 256 / kWarps;
+  E v[kN];
+  if (!tr) {   // c = warp + kWarps kc, r = lane + 32 kr
 #pragma unroll
-    for (int kc = 0; kc < 4; ++kc) {
+    for (int kc = 0; kc < kN / 8; ++kc) {
 #pragma unroll
       for (int kr = 0; kr < 8; ++kr) {
-        const int c = warp + 8 * kc, r = lane + 32 * kr;
+        const int c = warp + kWarps * kc, r = lane + 32 * kr;
         v[kc * 8 + kr] = (c < cols && r < rows) ? masked_ld(g, r0 + r, c0 + c, nb, tr, mask) : E(0);
       }
     }
 #pragma unroll
-    for (int kc = 0; kc < 4; ++kc) {
+    for (int kc = 0; kc < kN / 8; ++kc) {
 #pragma unroll
       for (int kr = 0; kr < 8; ++kr) {
-        const int c = warp + 8 * kc, r = lane + 32 * kr;
+        const int c = warp + kWarps * kc, r = lane + 32 * kr;
         if (c < cols && r < rows) put(s, hi, r * rs + c * cs, v[kc * 8 + kr]);
       }
     }
-  } else {     // r = warp + 8 kr, c = lane
+  } else {     // r = warp + kWarps kr, c = lane
 #pragma unroll
-    for (int kr = 0; kr < 32; ++kr) {
-      const int r = warp + 8 * kr;
+    for (int kr = 0; kr < kN; ++kr) {
+      const int r = warp + kWarps * kr;
       v[kr] = (lane < cols && r < rows) ? masked_ld(g, r0 + r, c0 + lane, nb, tr, mask) : E(0);
     }
 #pragma unroll
-    for (int kr = 0; kr < 32; ++kr) {
-      const int r = warp + 8 * kr;
+    for (int kr = 0; kr < kN; ++kr) {
+      const int r = warp + kWarps * kr;
       if (lane < cols && r < rows) put(s, hi, r * rs + lane * cs, v[kr]);
     }
   }
@@ -951,12 +953,13 @@ __device__ void apply_rm(const E* V, const E* Vh, int lv, int vrows, int kb, con
   }
   __syncthreads();
   // phase 2: W2 = op(T) W, then Ct -= W2.  For kb = 32 and ncols = 32 each thread takes the rows
-  // g, 31 - g, g + 8, 23 - g of one column (g = warp), so that every thread does 66 FMAs.
+  // g, 31 - g, g + 8, 23 - g (with 16 warps the first two) of one column (g = warp), so that every thread does
+  // 66 (33) FMAs.
   if (kb == 32 && ncols == 32) {
     const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
     const int arow[4] = {g, 31 - g, g + 8, 23 - g};
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 32 / kWarps; ++q) {
       const int a = arow[q];
       E s = E(0);
       if (!notrans) {
@@ -1003,8 +1006,8 @@ __device__ void apply_rm(const E* V, const E* Vh, int lv, int vrows, int kb, con
 // ---------------------------------------------------------------------------------------------
 struct Umma {
   uint32_t tmem;      // TMEM base address of this CTA's allocation
-  uint32_t mbar;      // shared-memory address of the completion mbarrier
-  uint32_t phase;     // parity of the next completion
+  uint32_t mbar;      // shared-memory address of the completion mbarriers (four: the FP32 path uses the first)
+  uint32_t phase;     // parity of the next completion (bit i: mbarrier i)
   uint32_t ncols_alloc;
   int failed;         // a completion wait ran out (the MMAs may still be in flight)
 };
@@ -1514,12 +1517,15 @@ __device__ __forceinline__ bool run_update(unsigned char* smb, int type, const E
     if (prm.f32_simt == 0 &&
         task_update_umma(smb, type, X, Cp, C, tr, notrans, Tg, nb, ib, w, blk0, blk1, col0, ncols, um, prm))
       return true;
-  } else if constexpr (kDig) {
+  }
+#if BD_EXEC_PART == 1
+  if constexpr (kDig) {
     if (um.ncols_alloc >= kDigTmem && digits_fit(nb, ib, ncols))
       done = task_update_digits(smb, type, X, Cp, C, tr, notrans, Tg, nb, ib, blk0, blk1, col0, ncols, um, prm);
     if (done == blk1 - blk0) return true;
     if (notrans) blk1 -= done; else blk0 += done;
   }
+#endif
   task_update(smb, type, X, Cp, C, tr, notrans, Tg, nb, ib, w, blk0, blk1, col0, ncols, prm.f32_simt == 1);
   return done > 0;
 }
@@ -1786,7 +1792,7 @@ __device__ void task_bwd_panel(unsigned char* smb, int kind, const E* X, E* A_s,
   // of FP64 operations on one thread is slow): the eight warp partials are combined by a 3-level
   // shuffle, and the divisions by beta_k and beta_k tau_k are replaced by reciprocals formed up front
   // for all k in parallel (beta_k, the top entry of column k, is not changed before step k).
-  static_assert(kWarps == 8, "warp-partial reductions assume 8 warps");
+  static_assert(kWarps == 8 || sizeof(E) == 0, "warp-partial reductions assume 8 warps");
   double* sc = rsc + kWarps;       // sc[0..3]: om, tau_bar, -1 / (beta tau), -beta_bar tau
   double* wbp = rsc + 16;          // per warp: sum_j wsA_j bA_j over its columns
   double* vbp = rsc + 24;          // per warp: v_bar . v
@@ -2030,10 +2036,10 @@ __device__ int next_task(const ExecParams& prm) {
 // 2.37 ms against 2.44).
 template <typename E, bool kBwd, bool kDig>
 __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm) {
-  extern __shared__ __align__(128) unsigned char smb[];
+  extern __shared__ __align__(kSmemAlign) unsigned char smb[];
   __shared__ int s_idx;
   __shared__ int s_abort;
-  __shared__ __align__(8) uint64_t s_mbar;
+  __shared__ __align__(8) uint64_t s_mbar[4];
   __shared__ uint32_t s_tmem;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // TMEM columns for the tcgen05 phases of the updates, held for the whole launch (the host enables it
@@ -2048,14 +2054,15 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
       }
       if (threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar)) : "memory");
+        for (int i = 0; i < 4; ++i)
+          asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(s_mbar + i)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncthreads();
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       um.tmem = s_tmem;
-      um.mbar = smem_u32(&s_mbar);
+      um.mbar = smem_u32(s_mbar);
       um.ncols_alloc = (uint32_t)prm.umma_cols;
     }
   }
@@ -2477,7 +2484,7 @@ size_t umma_smem_bytes(int nb, int ib, int w) {
 }
 
 int digits_tmem(int nb, int ib, int w) { return digits_fit(nb, ib, w < nb ? w : nb) ? kDigTmem : 0; }
-size_t digits_smem_bytes() { return kHeaderDoubles * sizeof(double) + kDigBytes; }
+size_t digits_smem_bytes() { return kDigBytes; }
 
 size_t bwd_smem_bytes(int nb, int ib, int hw, int esize) {
   const BwdLayout a = layout_bwd_update(nb, ib, hw, esize), b = layout_bwd_panel(nb, ib, esize);
@@ -2518,14 +2525,14 @@ cudaError_t exec_set_smem(size_t smem, int esize, bool bwd, bool digits) {
 
 int exec_max_ctas_per_sm(size_t smem, int esize, bool bwd, bool digits) {
   int n = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, exec_fn(esize, bwd, digits), kThreads, smem);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, exec_fn(esize, bwd, digits), digits ? kThreadsDigits : kThreads, smem);
   return e == cudaSuccess ? n : 0;
 }
 
 cudaError_t launch_exec(const ExecParams& prm, int grid, size_t smem, cudaStream_t st) {
   void* args[1] = {const_cast<ExecParams*>(&prm)};
-  return cudaLaunchKernel(exec_fn(prm.esize, prm.bwd.part != nullptr, prm.umma_cols > 0), dim3((unsigned)grid), dim3(kThreads), args, smem,
-                          st);
+  return cudaLaunchKernel(exec_fn(prm.esize, prm.bwd.part != nullptr, prm.umma_cols > 0), dim3((unsigned)grid),
+                          dim3(prm.esize == 8 && prm.umma_cols > 0 ? kThreadsDigits : kThreads), args, smem, st);
 }
 
 cudaError_t launch_pack_batched(const PackDesc* d, int count, int64_t total_tiles, int esize, cudaStream_t st) {

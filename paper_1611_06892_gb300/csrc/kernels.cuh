@@ -7,7 +7,13 @@
 
 namespace bd {
 
-constexpr int kThreads = 256;       // threads of every executor CTA
+// Threads of an executor CTA: 512 for the FP64 instantiation with digit products (BD_EXEC_PART 1), else 256.
+constexpr int kThreadsDigits = 512;
+#if defined(BD_EXEC_PART) && BD_EXEC_PART == 1
+constexpr int kThreads = kThreadsDigits;
+#else
+constexpr int kThreads = 256;
+#endif
 constexpr int kMaxNb = 256;
 
 // Error word layout written by the executor: err[0] = code (0 ok, 1 wait ran out, 2 bad task),

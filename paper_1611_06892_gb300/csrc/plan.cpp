@@ -512,11 +512,12 @@ inline int32_t make_op(int type, bool tr, bool notrans, int strip, int blk, int 
 // ib 32; FP32 storage at 8192^2 with the tcgen05 updates, FP64 at 4096^2).  Mode 0 is the flop count
 // alone, with FP32-storage panel factors counted twice.
 enum WeightClass { W_PF_GE, W_PF_TS, W_PF_TT, W_PU_GE, W_PU_TS, W_PU_TT, W_UNMQR, W_TSMQR, W_TTMQR };
-static int64_t prio_weight(int64_t flops, int cls, int esize, int mode) {
+static int64_t prio_weight(int64_t flops, int cls, int esize, int mode, bool digits) {
   static const int64_t kF32[9] = {640, 400, 650, 125, 115, 210, 135, 100, 150};
   static const int64_t kF64[9] = {71, 51, 74, 71, 70, 79, 117, 100, 119};
+  static const int64_t kDig[9] = {645, 470, 690, 183, 115, 171, 174, 100, 182};   // FP64, digit products (8192^2)
   if (mode == 0) return (cls <= W_PF_TT && esize == 4 ? 2 : 1) * flops;
-  return std::max<int64_t>(1, flops * (esize == 4 ? kF32[cls] : kF64[cls]) / 100);
+  return std::max<int64_t>(1, flops * (esize == 4 ? kF32[cls] : (digits ? kDig[cls] : kF64[cls])) / 100);
 }
 
 void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int variant, int64_t R, int strip_w,
@@ -571,6 +572,7 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
   std::vector<int32_t> panel_last(nt, -1);   // last sub-task of each panel task
   std::vector<int64_t> rd, wr;
   const int64_t ib2 = (int64_t)ib * ib;
+  const bool digits = esize == 8 && digits_fit(nb, ib, w);
 
   auto tref = [&](int buf, int oa, int ob, bool lq) {
     const int x = lq ? ob : oa, y = lq ? oa : ob;
@@ -611,7 +613,7 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
         wr.push_back(it.t(slot, b));
         const int64_t rows = kind == PK_GE ? nb - (int64_t)b * ib : (kind == PK_TS ? nb : (int64_t)(b + 1) * ib);
         d.op = make_op(PF, lq, false, 0, b, kind);
-        last = g.add(d, prio_weight(12 * ib2 * rows, W_PF_GE + kind, esize, prio), rd, wr, -1);
+        last = g.add(d, prio_weight(12 * ib2 * rows, W_PF_GE + kind, esize, prio, digits), rd, wr, -1);
         // PU(b, s)
         for (int s = b + 1; s < nblk; ++s) {
           rd.clear();
@@ -632,7 +634,7 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
           }
           rd.push_back(it.t(slot, b));
           d.op = make_op(PU, lq, false, s, b, kind);
-          last = g.add(d, prio_weight(6 * ib2 * rows, W_PU_GE + kind, esize, prio), rd, wr, -1);
+          last = g.add(d, prio_weight(6 * ib2 * rows, W_PU_GE + kind, esize, prio, digits), rd, wr, -1);
         }
       }
       panel_last[x] = last;
@@ -657,7 +659,7 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
           }
         }
         d.op = make_op(t.type, lq, false, s, 0, 0);
-        g.add(d, prio_weight(per_strip, t.type == UNMQR ? W_UNMQR : (t.type == TSMQR ? W_TSMQR : W_TTMQR), esize, prio),
+        g.add(d, prio_weight(per_strip, t.type == UNMQR ? W_UNMQR : (t.type == TSMQR ? W_TSMQR : W_TTMQR), esize, prio, digits),
               rd, wr, panel_last[owner]);
       }
     } else {   // COPY(i, j): R part of A's tile (i, j) into the second phase's tile (i, j)

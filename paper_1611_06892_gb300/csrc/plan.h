@@ -57,6 +57,20 @@ struct DevTask {
   int32_t flags;     // bit 0: diagonal COPY (upper triangle only); bits 8-31: matrix of a batch
 };
 
+#ifdef __CUDACC__
+#define BD_HD __host__ __device__
+#else
+#define BD_HD
+#endif
+// Whether an FP64 block update of these sizes (ncols columns of an nb tile, ib reflectors) runs as digit products on
+// tcgen05 (update_digits.cuh).  Its cost per block of reflectors hardly depends on the sizes (10 us at nb 64, 13 us at
+// 256 for 32 columns), that on the FP64 units is nb x ib x columns: they cross near nb x ib = 1024 (nb 64, ib 16: 51 us a
+// strip against 75; nb 32, ib 8: 45 against 40).
+constexpr int kDigitRows = 256;
+BD_HD inline bool digits_fit(int nb, int ib, int ncols) {
+  return nb % 8 == 0 && nb <= kDigitRows && ib % 8 == 0 && ib <= 32 && ncols % 8 == 0 && ncols <= 32 && nb * ib >= 1024;
+}
+
 inline int32_t tile_ref(int buf, int64_t idx) { return (int32_t)(((uint32_t)buf << 28) | (uint32_t)idx); }
 
 struct Plan {
