@@ -532,7 +532,7 @@ int band_impl(bidiag_handle h, int64_t m, int64_t n, const E* d_A, int64_t lda, 
   rc = run_exec(h, *pd, (int)pd->plan.dev.size(), r->tiles, (int64_t)r->p * r->q, r->tiles2,
                 r->tiles2 ? (int64_t)r->q * r->q : 0, nullptr, 0, r->T, pd->plan.npanels, nb, ib, w, (int)sizeof(E),
                 timed, nullptr, 0, 0, nullptr, nullptr, nullptr,
-                (sizeof(E) == 8 && !r->tiles2) ? bd::kWindowF64BiDiag : 0);
+                (sizeof(E) == 8 && !r->tiles2 && !bd::digits_fit(nb, ib, w)) ? bd::kWindowF64BiDiag : 0);
   h->timed = timed;
   if (rc) return bail(rc);
   if (tiles2 && variant != BIDIAG_RBIDIAG) {

@@ -621,12 +621,62 @@ __device__ void factor_panel(int mode, E* P, int lp, int rows, int kb, E* Rt, in
   __syncthreads();
 }
 
+// T from the reflectors' tau and the strict upper part of G = V^T V (kb x kb, ld kb; kb x kb more are scratch): the
+// inverse of the upper triangular matrix with diagonal 1 / tau and G above it.  The forward recurrence
+// T[l,l] = tau_l, T[0:l, l] = -tau_l T[0:l, 0:l] G[0:l, l] inside diagonal blocks of 8 columns (all blocks at once),
+// then blocks are merged pairwise, [T11 T12; 0 T22] with T12 = -T11 G12 T22 (the product of two compact WY blocks),
+// so the sequential depth is 8 + 2 log2(kb/8) barrier steps instead of kb.
+template <typename E>
+__device__ void t_from_gram(int kb, const double* tau_s, E* Tb, int ldt, E* G) {
+  E* Y = G + kb * kb;
+  constexpr int kB0 = 8;
+  for (int o = threadIdx.x; o < kb * kb; o += kThreads) Tb[(o % kb) + (o / kb) * ldt] = E(0);
+  __syncthreads();
+  // diagonal blocks of kB0 columns: the forward recurrence, all blocks in parallel
+  const int nblk0 = (kb + kB0 - 1) / kB0;
+  for (int step = 0; step < kB0; ++step) {
+    for (int u = threadIdx.x; u < nblk0 * kB0; u += kThreads) {
+      const int d = u / kB0, a = d * kB0 + u % kB0, l = d * kB0 + step;
+      if (l >= kb || a > l) continue;
+      if (a == l) {
+        Tb[l + l * ldt] = (E)tau_s[l];
+      } else {
+        E acc = E(0);
+        for (int t = a; t < l; ++t) acc += Tb[a + t * ldt] * G[t + l * kb];
+        Tb[a + l * ldt] = -(E)tau_s[l] * acc;
+      }
+    }
+    __syncthreads();
+  }
+  // pairwise merges: T12 = -T11 (G12 T22) for blocks [c0, c0 + h) and [c0 + h, c1)
+  for (int h = kB0; h < kb; h *= 2) {
+    const int npair = (kb + 2 * h - 1) / (2 * h);
+    for (int u = threadIdx.x; u < npair * h * h; u += kThreads) {     // Y = G12 T22
+      const int pr = u / (h * h), i = (u % (h * h)) % h, j = (u % (h * h)) / h;
+      const int c0 = pr * 2 * h, c1 = min(c0 + 2 * h, kb);
+      if (c0 + h + j >= c1) continue;
+      const int col = c0 + h + j;
+      E acc = E(0);
+      for (int t = c0 + h; t <= col; ++t) acc += G[(c0 + i) + t * kb] * Tb[t + col * ldt];
+      Y[(c0 + i) + col * kb] = acc;
+    }
+    __syncthreads();
+    for (int u = threadIdx.x; u < npair * h * h; u += kThreads) {     // T12 = -T11 Y
+      const int pr = u / (h * h), i = (u % (h * h)) % h, j = (u % (h * h)) / h;
+      const int c0 = pr * 2 * h, c1 = min(c0 + 2 * h, kb);
+      if (c0 + h + j >= c1) continue;
+      const int row = c0 + i, col = c0 + h + j;
+      E acc = E(0);
+      for (int t = row; t < c0 + h; ++t) acc += Tb[row + t * ldt] * Y[t + col * kb];
+      Tb[row + col * ldt] = -acc;
+    }
+    __syncthreads();
+  }
+}
+
 // T factor (kb x kb, upper) of the kb reflectors in P, Q = H_0 ... H_{kb-1} = I - V T V^T.  G is
 // 2 kb x kb scratch (the Gram matrix V^T V, then a work block).  The Gram entries are computed in 2 x 2
-// blocks per thread (no cross-lane reductions).  T itself: the forward recurrence T[l,l] = tau_l,
-// T[0:l, l] = -tau_l T[0:l, 0:l] G[0:l, l] inside diagonal blocks of 8 columns (all blocks at once),
-// then blocks are merged pairwise, [T11 T12; 0 T22] with T12 = -T11 G12 T22 (the product of two compact
-// WY blocks), so the sequential depth is 8 + 2 log2(kb/8) barrier steps instead of kb.
+// blocks per thread (no cross-lane reductions).
 template <typename E>
 __device__ void build_t(int mode, const E* P, int lp, int rows, int kb, int voff, const double* tau_s, E* Tb, int ldt,
                         E* G) {
@@ -674,50 +724,7 @@ __device__ void build_t(int mode, const E* P, int lp, int rows, int kb, int voff
     if (a1 < l1 && a1 != a0 && l1 != l0) G[a1 + l1 * kb] = s11;
   }
   __syncthreads();
-  E* Y = G + kb * kb;
-  constexpr int kB0 = 8;
-  for (int o = threadIdx.x; o < kb * kb; o += kThreads) Tb[(o % kb) + (o / kb) * ldt] = E(0);
-  __syncthreads();
-  // diagonal blocks of kB0 columns: the forward recurrence, all blocks in parallel
-  const int nblk0 = (kb + kB0 - 1) / kB0;
-  for (int step = 0; step < kB0; ++step) {
-    for (int u = threadIdx.x; u < nblk0 * kB0; u += kThreads) {
-      const int d = u / kB0, a = d * kB0 + u % kB0, l = d * kB0 + step;
-      if (l >= kb || a > l) continue;
-      if (a == l) {
-        Tb[l + l * ldt] = (E)tau_s[l];
-      } else {
-        E acc = E(0);
-        for (int t = a; t < l; ++t) acc += Tb[a + t * ldt] * G[t + l * kb];
-        Tb[a + l * ldt] = -(E)tau_s[l] * acc;
-      }
-    }
-    __syncthreads();
-  }
-  // pairwise merges: T12 = -T11 (G12 T22) for blocks [c0, c0 + h) and [c0 + h, c1)
-  for (int h = kB0; h < kb; h *= 2) {
-    const int npair = (kb + 2 * h - 1) / (2 * h);
-    for (int u = threadIdx.x; u < npair * h * h; u += kThreads) {     // Y = G12 T22
-      const int pr = u / (h * h), i = (u % (h * h)) % h, j = (u % (h * h)) / h;
-      const int c0 = pr * 2 * h, c1 = min(c0 + 2 * h, kb);
-      if (c0 + h + j >= c1) continue;
-      const int col = c0 + h + j;
-      E acc = E(0);
-      for (int t = c0 + h; t <= col; ++t) acc += G[(c0 + i) + t * kb] * Tb[t + col * ldt];
-      Y[(c0 + i) + col * kb] = acc;
-    }
-    __syncthreads();
-    for (int u = threadIdx.x; u < npair * h * h; u += kThreads) {     // T12 = -T11 Y
-      const int pr = u / (h * h), i = (u % (h * h)) % h, j = (u % (h * h)) / h;
-      const int c0 = pr * 2 * h, c1 = min(c0 + 2 * h, kb);
-      if (c0 + h + j >= c1) continue;
-      const int row = c0 + i, col = c0 + h + j;
-      E acc = E(0);
-      for (int t = row; t < c0 + h; ++t) acc += Tb[row + t * ldt] * Y[t + col * kb];
-      Tb[row + col * ldt] = -acc;
-    }
-    __syncthreads();
-  }
+  t_from_gram(kb, tau_s, Tb, ldt, G);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1505,6 +1512,7 @@ __device__ bool task_update_umma(unsigned char* smb, int type, const float* X, f
 }
 
 #include "update_digits.cuh"
+#include "panel_digits.cuh"
 
 // An update (strip or panel block, arguments as task_update) on the tensor cores where the CTA holds TMEM for it
 // and the sizes fit, on the FMA units otherwise; true if any of it ran on tcgen05.
@@ -2147,9 +2155,15 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
     switch (type) {
       case PF: {
         E* A = (kind == PM_GE) ? nullptr : tile_ptr<E>(prm, mv, t.a, ok);
-        if (ok && Tg && blk < nblk && kind <= PM_TT)
-          task_panel_factor(smb, kind, X, A, tr, Tg, nb, ib, blk, prm.f32_scalars64 == 0);
-        else ok = false;
+        if (ok && Tg && blk < nblk && kind <= PM_TT) {
+#if BD_EXEC_PART == 1
+          if (um.ncols_alloc >= kDigTmem && digits_fit(nb, ib, ib))
+            on_tc5 = task_panel_digits(smb, kind, X, A, tr, Tg, nb, ib, blk, um, prm);
+#endif
+          if (!on_tc5) task_panel_factor(smb, kind, X, A, tr, Tg, nb, ib, blk, prm.f32_scalars64 == 0);
+        } else {
+          ok = false;
+        }
         break;
       }
       case PU: {

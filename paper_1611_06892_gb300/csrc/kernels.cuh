@@ -52,8 +52,9 @@ struct BwdParams {
 };
 
 // Executor look-ahead of one-matrix FP64 BiDiag reductions (queue entries scanned for a ready sub-task):
-// 8192^2 1374 -> 1330 ms, 4096^2 232 -> 222 ms against strict queue order; FP32 storage, R-BiDiag and
-// batches were not faster with it and keep strict order.
+// 8192^2 1374 -> 1330 ms, 4096^2 232 -> 222 ms against strict queue order with sub-tasks on the FP64 units; FP32
+// storage, R-BiDiag, batches and the ten times shorter sub-tasks of the digit products (8192^2 196.6 ms in strict
+// order, 203.1 with the window) were not faster with it and keep strict order.
 constexpr int kWindowF64BiDiag = 1024;
 
 struct ExecParams {

@@ -515,7 +515,7 @@ enum WeightClass { W_PF_GE, W_PF_TS, W_PF_TT, W_PU_GE, W_PU_TS, W_PU_TT, W_UNMQR
 static int64_t prio_weight(int64_t flops, int cls, int esize, int mode, bool digits) {
   static const int64_t kF32[9] = {640, 400, 650, 125, 115, 210, 135, 100, 150};
   static const int64_t kF64[9] = {71, 51, 74, 71, 70, 79, 117, 100, 119};
-  static const int64_t kDig[9] = {645, 470, 690, 183, 115, 171, 174, 100, 182};   // FP64, digit products (8192^2)
+  static const int64_t kDig[9] = {277, 124, 205, 183, 115, 171, 174, 100, 183};   // FP64, digit products (8192^2)
   if (mode == 0) return (cls <= W_PF_TT && esize == 4 ? 2 : 1) * flops;
   return std::max<int64_t>(1, flops * (esize == 4 ? kF32[cls] : (digits ? kDig[cls] : kF64[cls])) / 100);
 }

@@ -123,15 +123,15 @@ __device__ __forceinline__ void digit_pair(int64_t x0, int64_t x1, uint32_t* w) 
   for (int j = 0; j < ND; ++j)               // minus 1152: the signed digit
     asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(w[j]) : "r"(r[j]), "r"(0x64806480u));
 }
-// Digits of eight values of row r, columns 8 g .. 8 g + 7, into an operand at sm.
-__device__ __forceinline__ void put_digits(unsigned char* sm, int r, int g, const int64_t* x) {
+// Digits of eight values of row r, columns 8 g .. 8 g + 7, into an operand at sm (slice: bytes of one digit).
+__device__ __forceinline__ void put_digits(unsigned char* sm, int r, int g, const int64_t* x, int slice = kDigSlice) {
   uint32_t w[4][kDigN];
 #pragma unroll
   for (int p = 0; p < 4; ++p) digit_pair<kDigN>(x[2 * p], x[2 * p + 1], w[p]);
   unsigned char* o = sm + r * 64 + ((g ^ ((r >> 1) & 3)) << 4);
 #pragma unroll
   for (int j = 0; j < kDigN; ++j)
-    *reinterpret_cast<uint4*>(o + j * kDigSlice) = make_uint4(w[0][j], w[1][j], w[2][j], w[3][j]);
+    *reinterpret_cast<uint4*>(o + j * slice) = make_uint4(w[0][j], w[1][j], w[2][j], w[3][j]);
 }
 // Descriptor of an operand in the digit layout (64-byte swizzle): stride of 32-column slices (M/N-major), and of
 // groups of 8 rows (512 bytes).
@@ -152,6 +152,82 @@ __device__ __forceinline__ float transpose_sum16(float* v) {
     }
   }
   return v[0] + __shfl_xor_sync(kFull, v[0], 16);
+}
+
+// E_c of the columns whose entries the CTA's threads hold as FP64 bit patterns (thread: 16 columns of a row of x and of
+// a row of y): into colE, and that of column lane % 16 of the thread's half into *E.  Two passes: the largest exponent
+// of a column, then the sum of its squares scaled by it.  False (for all) if a column is out of range, or zero and
+// zero_ok is false.
+__device__ __forceinline__ bool column_exponents(const int64_t* cf, const int64_t* cq, int* colE, uint32_t* red, int* E,
+                                                 bool zero_ok = true) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ch = threadIdx.x >> 8;
+  uint32_t mymax = 0;
+#pragma unroll
+  for (int c = 0; c < 16; ++c) {
+    const uint32_t h0 = (uint32_t)(cf[c] >> 32) & 0x7fffffffu, h1 = (uint32_t)(cq[c] >> 32) & 0x7fffffffu;
+    const uint32_t nz = min((uint32_t)cf[c] | (uint32_t)cq[c], 1u);
+    const uint32_t m = __reduce_max_sync(kFull, max(max(h0, h1), nz));
+    if ((lane & 15) == c) mymax = m;
+  }
+  if (lane < 16) red[warp * 16 + lane] = mymax;
+  __syncthreads();
+  uint32_t mx = 0;                  // of column cb + (lane & 15)
+#pragma unroll
+  for (int q = 0; q < 8; ++q) mx = max(mx, red[(8 * ch + q) * 16 + (lane & 15)]);
+  const int emax = (int)(mx >> 20);
+  if (__syncthreads_or(mx == 0 ? !zero_ok : (emax < 64 || emax > 2000))) return false;
+  float sq[16];
+#pragma unroll
+  for (int c = 0; c < 16; ++c) {
+    const int base = (__shfl_sync(kFull, emax, c) - 120) * (1 << 20);
+    const int d0 = max((int)((uint32_t)(cf[c] >> 32) & 0x7fffffffu) - base, 0);
+    const int d1 = max((int)((uint32_t)(cq[c] >> 32) & 0x7fffffffu) - base, 0);
+    const float f0 = __int_as_float(d0 << 3), f1 = __int_as_float(d1 << 3);   // |x| 2^(1016 - emax), truncated
+    sq[c] = f0 * f0 + f1 * f1;
+  }
+  const float part = transpose_sum16(sq);
+  if (lane < 16) red[warp * 16 + lane] = __float_as_uint(part);
+  __syncthreads();
+  float s2 = 0.0f;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) s2 += __uint_as_float(red[(8 * ch + q) * 16 + (lane & 15)]);
+  const int k = (int)(__float_as_uint(sqrtf(s2) * 1.03f) >> 23) - 127;
+  *E = mx == 0 ? 0 : k + 1 + emax - 1016;
+  if ((warp & 7) == 0 && lane < 16) colE[16 * ch + lane] = *E;
+  return true;
+}
+
+// Readout of the digit products of phase 1 (lane = (digit j of A, column of A), column = (digit i of B, column of B)):
+// P[q][a][c] += over the digits j = q and q + 4 of A, in units where the pair of leading digits weighs 2^(s + 24).
+// kWide: sums may exceed 2^22 (more than 256 rows).
+template <bool kWide>
+__device__ __forceinline__ void gram_partials(int64_t* P, uint32_t tq, int s) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp & 3;
+  const int sH = s - 8 * q, sL = 32 - s + 8 * q;
+  auto val = [](uint32_t f) { return kWide ? __float2int_rn(__uint_as_float(f)) : int_of(f); };
+#pragma unroll 1
+  for (int cg = (warp >> 2) * 8, ce = cg + 8; cg < ce; cg += 4) {
+    uint32_t d[7][4], e[4][4];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) tmem_ld4(tq + 32 * i + cg, d[i]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) tmem_ld4(tq + 256 + 32 * i + cg, e[i]);
+    tmem_wait_ld();
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      // digit pairs with i + j >= 8 are left out: i <= 7 - q of the first block, i <= 3 - q of the second
+      const int64_t H = wide(val(d[0][c]) * 256 + val(d[1][c]), 65536, val(d[2][c]) * 256 + val(d[3][c]));
+      int l4 = val(d[4][c]), l5 = 0, l6 = 0, l7 = 0;
+      if (q < 3) {
+        l4 += val(e[0][c]);
+        l5 = val(d[5][c]) + val(e[1][c]);
+      }
+      if (q < 2) l6 = val(d[6][c]) + val(e[2][c]);
+      if (q < 1) l7 = val(e[3][c]);
+      const int64_t L = wide(l4, 1 << 24, wide(l5, 1 << 16, wide(l6, 256, l7)));
+      P[(q * 32 + lane) * 33 + cg + c] = (int64_t)((uint64_t)H << sH) + (L >> sL);
+    }
+  }
 }
 
 // task_update on the digit path: returns the number of blocks applied (from the first in the order of
@@ -247,47 +323,15 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
       }
     };
     load_row(C, own, cf);
-    // two passes over [Cp; C]: the largest exponent of a column, then the sum of squares scaled by it
     const bool ownp = top && r >= blk0 * ib && r < blk1 * ib;
     int64_t cq[16];
     load_row(Cp, ownp, cq);
-    uint32_t mymax = 0;
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const uint32_t h0 = (uint32_t)(cf[c] >> 32) & 0x7fffffffu, h1 = (uint32_t)(cq[c] >> 32) & 0x7fffffffu;
-      const uint32_t nz = min((uint32_t)cf[c] | (uint32_t)cq[c], 1u);
-      const uint32_t m = __reduce_max_sync(kFull, max(max(h0, h1), nz));
-      if ((lane & 15) == c) mymax = m;
-    }
-    if (lane < 16) red[warp * 16 + lane] = mymax;
-    __syncthreads();
-    uint32_t mx = 0;                  // of column cb + (lane & 15)
-#pragma unroll
-    for (int q = 0; q < 8; ++q) mx = max(mx, red[(8 * ch + q) * 16 + (lane & 15)]);
-    const int emax = (int)(mx >> 20);
-    if (__syncthreads_or(mx != 0 && (emax < 64 || emax > 2000))) {
+    int E;
+    if (!column_exponents(cf, cq, colE, red, &E)) {
       wait_v();
       __syncthreads();
       return 0;
     }
-    float sq[16];
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const int base = (__shfl_sync(kFull, emax, c) - 120) * (1 << 20);
-      const int d0 = max((int)((uint32_t)(cf[c] >> 32) & 0x7fffffffu) - base, 0);
-      const int d1 = max((int)((uint32_t)(cq[c] >> 32) & 0x7fffffffu) - base, 0);
-      const float f0 = __int_as_float(d0 << 3), f1 = __int_as_float(d1 << 3);   // |x| 2^(1016 - emax), truncated
-      sq[c] = f0 * f0 + f1 * f1;
-    }
-    const float part = transpose_sum16(sq);
-    if (lane < 16) red[warp * 16 + lane] = __float_as_uint(part);
-    __syncthreads();
-    float s2 = 0.0f;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) s2 += __uint_as_float(red[(8 * ch + q) * 16 + (lane & 15)]);
-    const int k = (int)(__float_as_uint(sqrtf(s2) * 1.03f) >> 23) - 127;
-    const int E = mx == 0 ? 0 : k + 1 + emax - 1016;
-    if ((warp & 7) == 0 && lane < 16) colE[cb + lane] = E;
 #pragma unroll
     for (int c = 0; c < 16; ++c) cf[c] = to_fixed(__longlong_as_double(cf[c]), 63 - __shfl_sync(kFull, E, c));
   }
@@ -401,35 +445,7 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
     }
     // ---- partial sums of W 2^(62 - E_c): lane = (digit j = q of V, reflector), 8 columns per warp -------
     int64_t* P = reinterpret_cast<int64_t*>(sm + kDigP);
-    {
-      const int q = warp & 3;
-      const int sH = 25 - 8 * q, sL = 7 + 8 * q;
-#pragma unroll 1
-      for (int cg = (warp >> 2) * 8, ce = cg + 8; cg < ce; cg += 4) {
-      uint32_t d[7][4], e[4][4];
-#pragma unroll
-      for (int i = 0; i < 7; ++i) tmem_ld4(tq + 32 * i + cg, d[i]);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) tmem_ld4(tq + 256 + 32 * i + cg, e[i]);
-      tmem_wait_ld();
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        // digit pairs with i + j >= 8 are left out: i <= 7 - q of the first block, i <= 3 - q of the second
-        constexpr uint32_t kOff = kMagicBits * 257u;
-        const int p01 = (int)(mag(d[0][c]) * 256 + mag(d[1][c]) - kOff), p23 = (int)(mag(d[2][c]) * 256 + mag(d[3][c]) - kOff);
-        const int64_t H = wide(p01, 65536, p23);
-        int l4 = int_of(d[4][c]), l5 = 0, l6 = 0, l7 = 0;
-        if (q < 3) {
-          l4 += int_of(e[0][c]);
-          l5 = int_of(d[5][c]) + int_of(e[1][c]);
-        }
-        if (q < 2) l6 = int_of(d[6][c]) + int_of(e[2][c]);
-        if (q < 1) l7 = int_of(e[3][c]);
-        const int64_t L = wide(l4, 1 << 24, wide(l5, 1 << 16, wide(l6, 256, l7)));
-        P[(q * 32 + lane) * 33 + cg + c] = (int64_t)((uint64_t)H << sH) + (L >> sL);
-      }
-      }
-    }
+    gram_partials<false>(P, tq, 25);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     if (!__syncthreads_and(ok ? 1 : 0)) {
       ok = false;
