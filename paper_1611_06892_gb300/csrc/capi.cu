@@ -64,7 +64,7 @@ struct BatchPlan {
   };
   std::vector<One> mats;
   std::vector<bd::MatInfo> info;
-  int64_t tot0 = 0, tot1 = 0, totT = 0, tiles_all = 0, cols_all = 0;
+  int64_t tot0 = 0, tot1 = 0, totT = 0, totV = 0, tiles_all = 0, cols_all = 0;
   size_t smem = 0;
   bool digits = false;          // FP64: some matrix's updates run as digit products
   int ntasks = 0;
@@ -111,6 +111,8 @@ struct bidiag_ctx {
   int f32_scalars64 = 0;           // FP32 storage: reflector scalars in FP64 instead of float pairs
   int window = -1;                 // executor look-ahead (queue entries scanned); -1: by precision and variant
   int prio = 1;                    // priority weights of the device program: 1 calibrated per kind, 0 flops
+  unsigned char* d_vd = nullptr;   // storage of published panel blocks kept between launches, and its bytes
+  int64_t vd_cap = 0;
   int64_t* d_trace = nullptr;      // per-task trace of the last traced reduction
   std::map<std::tuple<int, int, int, int64_t>, int> splits;   // best three-step split per (p, q, tree, R)
   std::map<std::vector<int64_t>, std::shared_ptr<BatchPlan>> batches;   // batch programs by shapes / options
@@ -184,12 +186,14 @@ int64_t resources_of(bidiag_handle h, int nb, int w, int esize) {
   return std::max<int64_t>(1, (int64_t)h->nsm * (esize == 4 ? 64 : w) / nb);
 }
 
+constexpr int64_t kVdKeep = (int64_t)2 << 30;
+
 // Executor launch of a program held in pd with the given buffers.
 int run_exec(bidiag_handle h, const PlanDev& pd, int ntasks, void* b0, int64_t n0, void* b1, int64_t n1, void* b2,
              int64_t n2, void* T, int npanels, int nb, int ib, int w, int esize, bool timed = false,
              const bd::MatInfo* d_mats = nullptr, int nmats = 0, size_t smem_batch = 0,
              const void* const* bx = nullptr, const int64_t* nx = nullptr, const bd::BwdParams* bwd = nullptr,
-             int auto_window = 0, bool digits_batch = false) {
+             int auto_window = 0, bool digits_batch = false, int64_t vd_bytes = 0) {
   if (ntasks == 0) return BIDIAG_OK;
   size_t smem = d_mats ? smem_batch : (bwd ? bd::bwd_smem_bytes(nb, ib, bwd->hw, esize) : bd::exec_smem_bytes(nb, ib, w, esize));
   // tcgen05 updates (FP32 forward, one CTA per SM): TMEM for one accumulator of N = max(w, ib) (rounded to
@@ -267,10 +271,35 @@ int run_exec(bidiag_handle h, const PlanDev& pd, int ntasks, void* b0, int64_t n
   }
   CK(h, cudaMemsetAsync(pd.d_done, 0, sizeof(int) * (size_t)pd.nflags, h->stream));
   CK(h, cudaMemsetAsync(h->d_ctrl, 0, sizeof(int), h->stream));
+  // published panel blocks live for the launch only.  Up to kVdKeep bytes of storage stay with the handle, whose
+  // launches are ordered on its stream (8192^2: 1.6 GB, 3 ms to map when the pool had been trimmed at a
+  // synchronisation); without memory for them the updates do without
+  const bool vd_kept = vd_bytes <= kVdKeep;
+  if (digits && vd_bytes > 0) {
+    if (vd_kept && h->vd_cap >= vd_bytes) {
+      prm.vd = h->d_vd;
+    } else {
+      if (vd_kept && h->d_vd) {
+        CK(h, cudaFreeAsync(h->d_vd, h->stream));
+        h->d_vd = nullptr;
+        h->vd_cap = 0;
+      }
+      if (cudaMallocAsync((void**)&prm.vd, (size_t)vd_bytes, h->stream) != cudaSuccess) {
+        cudaGetLastError();
+        prm.vd = nullptr;
+      } else if (vd_kept) {
+        h->d_vd = prm.vd;
+        h->vd_cap = vd_bytes;
+      }
+    }
+  }
   const int grid = std::min<int64_t>((int64_t)h->nsm * per_sm, ntasks);
-  if (timed) CK(h, cudaEventRecord(h->ev[0], h->stream));
-  CK(h, bd::launch_exec(prm, grid, smem, h->stream));
-  if (timed) CK(h, cudaEventRecord(h->ev[1], h->stream));
+  cudaError_t e = cudaSuccess;
+  if (timed) e = cudaEventRecord(h->ev[0], h->stream);
+  if (e == cudaSuccess) e = bd::launch_exec(prm, grid, smem, h->stream);
+  if (e == cudaSuccess && timed) e = cudaEventRecord(h->ev[1], h->stream);
+  if (prm.vd && !vd_kept) cudaFreeAsync(prm.vd, h->stream);
+  CK(h, e);
   return BIDIAG_OK;
 }
 
@@ -532,7 +561,8 @@ int band_impl(bidiag_handle h, int64_t m, int64_t n, const E* d_A, int64_t lda, 
   rc = run_exec(h, *pd, (int)pd->plan.dev.size(), r->tiles, (int64_t)r->p * r->q, r->tiles2,
                 r->tiles2 ? (int64_t)r->q * r->q : 0, nullptr, 0, r->T, pd->plan.npanels, nb, ib, w, (int)sizeof(E),
                 timed, nullptr, 0, 0, nullptr, nullptr, nullptr,
-                (sizeof(E) == 8 && !r->tiles2 && !bd::digits_fit(nb, ib, w)) ? bd::kWindowF64BiDiag : 0);
+                (sizeof(E) == 8 && !r->tiles2 && !bd::digits_fit(nb, ib, w)) ? bd::kWindowF64BiDiag : 0, false,
+                (int64_t)pd->plan.npanels * (nb / ib) * bd::digit_block_bytes(nb));
   h->timed = timed;
   if (rc) return bail(rc);
   if (tiles2 && variant != BIDIAG_RBIDIAG) {
@@ -813,7 +843,9 @@ int band_batched_impl(bidiag_handle h, int64_t count, const int64_t* m, const in
     mi.ib = pl.ib;
     mi.w = pl.strip_w;
     mi.npanels = pl.npanels;
-    mi.pad = 0;
+    mi.offV = bp->totV;
+    if (esize == 8 && bd::digits_fit(pl.nb, pl.ib, pl.ib))
+      bp->totV += (int64_t)pl.npanels * (pl.nb / pl.ib) * bd::digit_block_bytes(pl.nb);
     bp->tiles_all += mi.ntiles[0];
     bp->cols_all += n[b];
   }
@@ -904,7 +936,7 @@ int band_batched_impl(bidiag_handle h, int64_t count, const int64_t* m, const in
   }
   rc = run_exec(h, bp->prog, bp->ntasks, store->tiles, tiles_all, store->tiles2, tot1 ? 1 : 0, nullptr, 0, store->T,
                 0, 0, 1, 1, esize, timed, static_cast<const bd::MatInfo*>(bp->d_mats), (int)count, smem, nullptr, nullptr,
-                nullptr, 0, bp->digits);
+                nullptr, 0, bp->digits, bp->totV);
   if (rc) return bail(rc);
   h->timed = timed;
   e = bd::launch_extract_batched(d_ex, (int)count, cols_all, esize, h->stream);
@@ -1258,6 +1290,7 @@ int bidiag_destroy(bidiag_handle h) {
     r->h = nullptr;
   }
   h->live.clear();
+  if (h->d_vd) cudaFreeAsync(h->d_vd, h->stream);
   cudaStreamSynchronize(h->stream);
   h->cache.clear();
   if (h->d_ctrl) cudaFree(h->d_ctrl);

@@ -1013,7 +1013,7 @@ __device__ void apply_rm(const E* V, const E* Vh, int lv, int vrows, int kb, con
 // ---------------------------------------------------------------------------------------------
 struct Umma {
   uint32_t tmem;      // TMEM base address of this CTA's allocation
-  uint32_t mbar;      // shared-memory address of the completion mbarriers (four: the FP32 path uses the first)
+  uint32_t mbar;      // shared-memory address of the completion mbarriers (five: the FP32 path uses the first)
   uint32_t phase;     // parity of the next completion (bit i: mbarrier i)
   uint32_t ncols_alloc;
   int failed;         // a completion wait ran out (the MMAs may still be in flight)
@@ -1518,8 +1518,8 @@ __device__ bool task_update_umma(unsigned char* smb, int type, const float* X, f
 // and the sizes fit, on the FMA units otherwise; true if any of it ran on tcgen05.
 template <typename E, bool kDig>
 __device__ __forceinline__ bool run_update(unsigned char* smb, int type, const E* X, E* Cp, E* C, int tr, bool notrans, const E* Tg,
-                           int nb, int ib, int w, int blk0, int blk1, int col0, int ncols, Umma& um,
-                           const ExecParams& prm) {
+                           int nb, int ib, int w, int blk0, int blk1, int col0, int ncols, const unsigned char* vd,
+                           Umma& um, const ExecParams& prm) {
   int done = 0;
   if constexpr (sizeof(E) == 4) {
     if (prm.f32_simt == 0 &&
@@ -1529,7 +1529,8 @@ __device__ __forceinline__ bool run_update(unsigned char* smb, int type, const E
 #if BD_EXEC_PART == 1
   if constexpr (kDig) {
     if (um.ncols_alloc >= kDigTmem && digits_fit(nb, ib, ncols))
-      done = task_update_digits(smb, type, X, Cp, C, tr, notrans, Tg, nb, ib, blk0, blk1, col0, ncols, um, prm);
+      done = vd ? task_update_digits<true>(smb, type, X, Cp, C, tr, notrans, Tg, nb, ib, blk0, blk1, col0, ncols, vd, um, prm)
+                : task_update_digits<false>(smb, type, X, Cp, C, tr, notrans, Tg, nb, ib, blk0, blk1, col0, ncols, vd, um, prm);
     if (done == blk1 - blk0) return true;
     if (notrans) blk1 -= done; else blk0 += done;
   }
@@ -1948,7 +1949,7 @@ __device__ void task_copy(const E* src, E* dst, int nb, bool diag) {
 // Tile reference (buffer << 28 | tile index) -> address, with the matrix's offsets and tile size.
 struct MatView {
   int nb, ib, w, npanels;
-  int64_t off[6], offT, nt[6];
+  int64_t off[6], offT, offV, nt[6];
 };
 template <typename E>
 __device__ __forceinline__ E* tile_ptr(const ExecParams& prm, const MatView& mv, int32_t ref, bool& ok) {
@@ -2047,7 +2048,7 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
   extern __shared__ __align__(kSmemAlign) unsigned char smb[];
   __shared__ int s_idx;
   __shared__ int s_abort;
-  __shared__ __align__(8) uint64_t s_mbar[4];
+  __shared__ __align__(8) uint64_t s_mbar[5];
   __shared__ uint32_t s_tmem;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // TMEM columns for the tcgen05 phases of the updates, held for the whole launch (the host enables it
@@ -2062,7 +2063,7 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
       }
       if (threadIdx.x == 0) {
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 5; ++i)
           asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(s_mbar + i)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       }
@@ -2135,14 +2136,14 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
       const int mat = (t.flags >> 8) & 0xffffff;
       if (mat >= prm.nmats) {
         ok = false;
-        mv = MatView{prm.nb, prm.ib, prm.w, 0, {0, 0, 0, 0, 0, 0}, 0, {0, 0, 0, 0, 0, 0}};
+        mv = MatView{prm.nb, prm.ib, prm.w, 0, {0, 0, 0, 0, 0, 0}, 0, 0, {0, 0, 0, 0, 0, 0}};
       } else {
         const MatInfo mi = prm.mats[mat];
-        mv = MatView{mi.nb, mi.ib, mi.w, mi.npanels, {mi.off[0], mi.off[1], 0, 0, 0, 0}, mi.offT,
+        mv = MatView{mi.nb, mi.ib, mi.w, mi.npanels, {mi.off[0], mi.off[1], 0, 0, 0, 0}, mi.offT, mi.offV,
                      {mi.ntiles[0], mi.ntiles[1], 0, 0, 0, 0}};
       }
     } else {
-      mv = MatView{prm.nb, prm.ib, prm.w, prm.npanels, {0, 0, 0, 0, 0, 0}, 0,
+      mv = MatView{prm.nb, prm.ib, prm.w, prm.npanels, {0, 0, 0, 0, 0, 0}, 0, 0,
                    {prm.ntiles[0], prm.ntiles[1], prm.ntiles[2], prm.ntiles[3], prm.ntiles[4], prm.ntiles[5]}};
     }
     const int nb = mv.nb, ib = mv.ib, wst = mv.w;
@@ -2152,15 +2153,27 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
                 ? static_cast<E*>(prm.T) + mv.offT + (size_t)t.tslot * ib * nb
                 : nullptr;
     if constexpr (!kBwd) {
+    // published blocks of this sub-task's panel (Q^T programs of the digit instantiation)
+    unsigned char* vd = nullptr;
+    if constexpr (kDig) {
+      if (prm.vd && Tg && !notrans && digits_fit(nb, ib, ib))
+        vd = prm.vd + mv.offV + (int64_t)t.tslot * nblk * digit_block_bytes(nb);
+    }
     switch (type) {
       case PF: {
         E* A = (kind == PM_GE) ? nullptr : tile_ptr<E>(prm, mv, t.a, ok);
         if (ok && Tg && blk < nblk && kind <= PM_TT) {
 #if BD_EXEC_PART == 1
           if (um.ncols_alloc >= kDigTmem && digits_fit(nb, ib, ib))
-            on_tc5 = task_panel_digits(smb, kind, X, A, tr, Tg, nb, ib, blk, um, prm);
+            on_tc5 = task_panel_digits(smb, kind, X, A, tr, Tg, nb, ib, blk,
+                                       vd ? vd + blk * digit_block_bytes(nb) : nullptr, um, prm);
+          if (!on_tc5) {
+            task_panel_factor(smb, kind, X, A, tr, Tg, nb, ib, blk, false);
+            if (vd) publish_block(smb, kind, X, tr, Tg, nb, ib, blk, vd + blk * digit_block_bytes(nb));
+          }
+#else
+          task_panel_factor(smb, kind, X, A, tr, Tg, nb, ib, blk, prm.f32_scalars64 == 0);
 #endif
-          if (!on_tc5) task_panel_factor(smb, kind, X, A, tr, Tg, nb, ib, blk, prm.f32_scalars64 == 0);
         } else {
           ok = false;
         }
@@ -2170,7 +2183,8 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
         E* A = (kind == PM_GE) ? nullptr : tile_ptr<E>(prm, mv, t.a, ok);
         const int utype = kind == PM_GE ? UNMQR : (kind == PM_TS ? TSMQR : TTMQR);
         if (ok && Tg && blk < strip && strip < nblk && kind <= PM_TT)
-          on_tc5 = run_update<E, kDig>(smb, utype, X, A, X, tr, false, Tg, nb, ib, wst, blk, blk + 1, strip * ib, ib, um, prm);
+          on_tc5 = run_update<E, kDig>(smb, utype, X, A, X, tr, false, Tg, nb, ib, wst, blk, blk + 1, strip * ib, ib, vd, um,
+                                       prm);
         else
           ok = false;
         break;
@@ -2182,8 +2196,8 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
         E* C = tile_ptr<E>(prm, mv, t.c, ok);
         const int col0 = strip * wst;
         if (ok && Tg && col0 < nb)
-          on_tc5 = run_update<E, kDig>(smb, type, X, A, C, tr, notrans, Tg, nb, ib, wst, 0, nblk, col0, min(wst, nb - col0), um,
-                              prm);
+          on_tc5 = run_update<E, kDig>(smb, type, X, A, C, tr, notrans, Tg, nb, ib, wst, 0, nblk, col0, min(wst, nb - col0), vd,
+                                       um, prm);
         else
           ok = false;
         break;

@@ -26,7 +26,7 @@ struct MatInfo {
   int64_t offT;         // element offset of its T slots
   int64_t ntiles[2];
   int32_t nb, ib, w, npanels;
-  int64_t pad;
+  int64_t offV;         // byte offset of its published panel blocks
 };
 
 // Matrix b of a batched pack / extract.
@@ -81,6 +81,8 @@ struct ExecParams {
   int umma_cols;        // forward programs: TMEM columns each CTA allocates for the tcgen05 phases (0: none)
   int f32_scalars64;    // FP32 tiles only: 1 = reflector beta / tau / scale in FP64 instead of float pairs
   int window;           // queue entries from the head a CTA scans for a ready sub-task (0: strict queue order)
+  unsigned char* vd;    // FP64 reductions with digit products: published panel blocks (digit_block_bytes each, by T slot
+                        // and inner block; null: the updates make the digits of V themselves)
   BwdParams bwd;        // adjoint program only
 };
 

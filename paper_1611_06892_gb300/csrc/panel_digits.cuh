@@ -120,9 +120,10 @@ __device__ __forceinline__ void inverse32(const double* G, const double* d, doub
   }
 }
 
-// Factors inner block b of a panel task as task_panel_factor does; false: refused, nothing written.
+// Factors inner block b of a panel task as task_panel_factor does, and publishes it in vd if that is given; false:
+// refused, nothing written.
 __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, double* X, double* A, int tr, double* Tg, int nb,
-                                               int ib, int b, Umma& um, const ExecParams& prm) {
+                                               int ib, int b, unsigned char* vd, Umma& um, const ExecParams& prm) {
   if ((smem_u32(sm) & 511) || (kind == PM_GE && (b + 1) * ib == nb)) return false;
   int* colE = reinterpret_cast<int*>(sm + kDigHead);                     // E_c
   uint32_t* red = reinterpret_cast<uint32_t*>(sm + kDigHead + 128);      // reduction scratch of column_exponents, then:
@@ -231,6 +232,7 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
   auto fail = [&]() {
     if (tid == 0) atomicCAS(prm.err, 0, DERR_TIMEOUT);
     for (int i = 0; i < 3; ++i) mbar_wait(um.mbar + 8 * i, ((um.phase >> i) & 1u) ^ 1u, prm.wait_ns);
+    wait_image();
     __syncthreads();
     return true;
   };
@@ -371,8 +373,6 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
       cf[c] = cb + c < ti ? min(max((int64_t)__mul64hi(Bs[ti * 33 + cb + c] << 2, dinv[cb + c] << 2) << 4, -one), one)
                           : (cb + c == ti ? one + 1 : 0);
   }
-#pragma unroll
-  for (int g = 0; g < 2; ++g) put_digits(sm + kDigV, r, 2 * ch + g, cf + 8 * g);
   if (own && ok) {
 #pragma unroll
     for (int c = 0; c < 16; c += 2) {
@@ -380,6 +380,8 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
       const bool on = cb + c < kb, w0 = on && (ge ? d > 0 : (!tt || d <= 0)), w1 = on && (ge ? d > 1 : (!tt || d <= 1));
       double* p = X + toff(r, c0 + cb + c, nb, tr);
       const double x = from_fixed(cf[c], 62), y = from_fixed(cf[c + 1], 62);
+      cf[c] = to_fixed(x, 62);                            // V as it is stored
+      cf[c + 1] = to_fixed(y, 62);
       if (tr && w0 && w1) {
         __stcg(reinterpret_cast<double2*>(p), make_double2(x, y));
       } else {
@@ -388,8 +390,11 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
       }
     }
   }
+#pragma unroll
+  for (int g = 0; g < 2; ++g) put_digits(sm + kDigV, r, 2 * ch + g, cf + 8 * g);
   // ---- V^T V (2^61), tau, T ------------------------------------------------------------------------
   fence_sync();
+  if (vd) store_image(sm, vd, nb);
   gram(false);
   gram_partials<false>(P, tq, 25);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -404,6 +409,11 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
   inverse32(G, diag, Td, G + 1024);
   for (int o = tid; o < kb * kb; o += kThreads)
     stg(Tg + (size_t)c0 * ib + o, Td[kb == 32 ? o : o % kb + o / kb * 32]);
+  if (vd) {
+    const double t[2] = {Td[arow + lane * 32], Td[arow + 1 + lane * 32]};
+    publish_t(vd, nb, t, true, reinterpret_cast<uint32_t*>(colS + 96));
+    wait_image();
+  }
   __syncthreads();
   return true;
 }

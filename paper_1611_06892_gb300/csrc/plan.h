@@ -71,6 +71,11 @@ BD_HD inline bool digits_fit(int nb, int ib, int ncols) {
   return nb % 8 == 0 && nb <= kDigitRows && ib % 8 == 0 && ib <= 32 && ncols % 8 == 0 && ncols <= 32 && nb * ib >= 1024;
 }
 
+// A published panel block (update_digits.cuh): kDigitCount digits of V, 64 bytes a row, T and a header.
+constexpr int kDigitCount = 7, kDigitTBytes = 32 * 34 * 8;
+BD_HD inline int digit_image_rows(int nb) { return (nb + 15) & ~15; }
+BD_HD inline int64_t digit_block_bytes(int nb) { return (int64_t)kDigitCount * digit_image_rows(nb) * 64 + kDigitTBytes + 128; }
+
 inline int32_t tile_ref(int buf, int64_t idx) { return (int32_t)(((uint32_t)buf << 28) | (uint32_t)idx); }
 
 struct Plan {

@@ -48,6 +48,8 @@ static_assert(kDigW2 + 8 * 2048 <= kDigP + 4 * kDigPStride, "W2 digits fit besid
 static_assert(kDigT + 32 * 34 * 8 <= kDigHead, "T fits");
 static_assert((kDigW2 & 127) == 0, "operand alignment");
 constexpr int kDigTmem = 512;
+constexpr int kDigTBytes = 32 * 34 * 8;
+static_assert(kDigTBytes == kDigitTBytes && kDigN == kDigitCount, "published blocks");
 
 #if BD_EXEC_PART == 1
 __host__ __device__ constexpr uint32_t umma_idesc_f16(int m, int n, bool a_mn, bool b_mn) {
@@ -74,6 +76,9 @@ __device__ __forceinline__ void bulk_copy(void* dst, const void* src, int size, 
   asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
                "l"(src), "r"(size), "r"(mbar)
                : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint32_t mbar, int bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
 }
 constexpr int kIssueWarp = 12;       // of the second row half: the first half's warps go on during the MMAs
 __device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(kFull, x, 0); }
@@ -230,12 +235,89 @@ __device__ __forceinline__ void gram_partials(int64_t* P, uint32_t tq, int s) {
   }
 }
 
+// Published blocks: what the updates of a reduction read of a panel block instead of V and T, made once by its factor
+// sub-task (a strip spent 4.4k of its 24k cycles a block on V's digits).  Digits of V in the operand layout
+// (digit_image_rows(nb) rows, zeros outside the block), T 2^(56 - eT) split as the updates read it, then two
+// integers: whether |v| <= 1 and eT <= 12 hold, and eT.
+// Starts the copy of the V area (16 KB a digit) into block vd; wait_image before the sub-task ends.
+__device__ __forceinline__ void store_image(unsigned char* sm, unsigned char* vd, int nb) {
+  if ((int)uniform(threadIdx.x >> 5) == kIssueWarp) {
+    const int lane = threadIdx.x & 31, img = digit_image_rows(nb) * 64;
+    if (lane < kDigN) {
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(vd + lane * img),
+                   "r"(smem_u32(sm + kDigV + lane * kDigSlice)), "r"(img)
+                   : "memory");
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    }
+  }
+}
+__device__ __forceinline__ void wait_image() {
+  if ((int)uniform(threadIdx.x >> 5) == kIssueWarp) {
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    asm volatile("fence.proxy.async;" ::: "memory");
+  }
+}
+// T and the two integers; t: rows 2 warp, 2 warp + 1 of column lane, ok: the block's V is in range (any thread).
+__device__ __forceinline__ void publish_t(unsigned char* vd, int nb, const double* t, bool good, uint32_t* red) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t h = max((uint32_t)__double2hiint(t[0]) & 0x7fffffffu, (uint32_t)__double2hiint(t[1]) & 0x7fffffffu);
+  const uint32_t hm = __reduce_max_sync(kFull, h);
+  if (lane == 0) red[warp] = hm;
+  const bool v_ok = __syncthreads_and(good ? 1 : 0) != 0;
+  const int eT = max((int)(__reduce_max_sync(kFull, red[lane & 15]) >> 20) - 1022, 1);
+  int2* Ts = reinterpret_cast<int2*>(vd + kDigN * digit_image_rows(nb) * 64);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int64_t f = to_fixed(t[k], 63 - eT) >> 7;
+    const int x = (int)((f + (1 << 27)) >> 28);
+    __stcg(Ts + (2 * warp + k) * 34 + lane, make_int2(x, (int)(f - ((int64_t)x << 28))));
+  }
+  if (threadIdx.x == 0)
+    __stcg(reinterpret_cast<int2*>(vd + digit_block_bytes(nb) - 128), make_int2(v_ok && eT <= 12 ? 1 : 0, eT));
+}
+// Publishes a block that task_panel_factor has just written.
+__device__ __noinline__ void publish_block(unsigned char* sm, int kind, const double* X, int tr, const double* Tg, int nb,
+                                           int ib, int b, unsigned char* vd) {
+  const int tid = threadIdx.x, kb = ib, c0 = b * ib, r = tid & 255, cb = 16 * (tid >> 8);
+  const int r0 = kind == PM_GE ? c0 : 0, r1 = kind == PM_TT ? c0 + kb : nb;
+  bool good = true;
+  __syncthreads();
+#pragma unroll
+  for (int g = 0; g < 2; ++g) {
+    int64_t v[8];
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const int c = cb + 8 * g + a, d = r - (c0 + c);
+      double x = 0.0;
+      if (c < kb && r >= r0 && r < r1) {
+        if (kind == PM_TS || (kind == PM_GE ? d > 0 : d <= 0)) x = ldg(X + toff(r, c0 + c, nb, tr));
+        if (kind == PM_GE && d == 0) x = 1.0;
+      }
+      good = good && ((uint32_t)__double2hiint(x) & 0x7fffffffu) <= 0x3ff00000u;
+      v[a] = to_fixed(x, 62);
+    }
+    put_digits(sm + kDigV, r, (cb >> 3) + g, v);
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncthreads();
+  store_image(sm, vd, nb);
+  const int arow = 2 * (tid >> 5), lane = tid & 31;
+  double t[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) t[k] = (arow + k < kb && lane < kb) ? ldg(Tg + (size_t)c0 * ib + arow + k + lane * kb) : 0.0;
+  publish_t(vd, nb, t, good, reinterpret_cast<uint32_t*>(sm + kDigHead + 128));
+  wait_image();
+  __syncthreads();
+}
+
 // task_update on the digit path: returns the number of blocks applied (from the first in the order of
 // application; C and Cp are up to date for them), the rest being out of the path's range.  Arguments as
-// task_update.
+// task_update; kPre: vd holds the panel's published blocks (Q^T only), and X and Tg are not read.
+template <bool kPre>
 __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, const double* X, double* Cp, double* C,
                                                int tr, bool notrans, const double* Tg, int nb, int ib, int blk0,
-                                               int blk1, int col0, int ncols, Umma& um, const ExecParams& prm) {
+                                               int blk1, int col0, int ncols, const unsigned char* vd, Umma& um,
+                                               const ExecParams& prm) {
   static_assert(kThreads == 512, "two threads a row");
   if (smem_u32(sm) & 511) return 0;                                      // the swizzle's alignment
   int* colE = reinterpret_cast<int*>(sm + kDigHead);                     // E_c
@@ -250,6 +332,22 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
   auto blk_of = [&](int bb) { return notrans ? blk1 - 1 - bb : blk0 + bb; };
 
   const int uwarp = (int)uniform(warp);
+  // kPre: V digits of the next application into their place (whole halves of 128 rows: rows outside the block are zeros
+  // there), by bulk copies of one warp counted by the fourth mbarrier
+  const int img = digit_image_rows(nb) * 64;
+  auto load_image = [&](int b) {
+    const int c = b * ib, r0 = type == UNMQR ? c & 128 : 0, r1 = type == TTMQR ? c + kb : nb;
+    const int o = r0 * 64, size = min(((r1 + 127) & ~127) * 64, img) - o;
+    const unsigned char* src = vd + (size_t)b * digit_block_bytes(nb);
+    asm volatile("fence.proxy.async;" ::: "memory");
+    if (lane == 0) mbar_expect(um.mbar + 24, kDigN * size);
+    __syncwarp();
+    if (lane < kDigN) bulk_copy(sm + kDigV + lane * kDigSlice + o, src + lane * img + o, size, um.mbar + 24);
+  };
+  auto load_head = [&](int b) {
+    return __ldcg(reinterpret_cast<const int2*>(vd + (size_t)(b + 1) * digit_block_bytes(nb) - 128));
+  };
+  int2 head = make_int2(1, 0);       // published block: whether it is in range, exponent of T
   // V block of the next application, as stored, into the staging area: columns (ld 256) for tr = 0, by bulk copies
   // of one warp counted by the fourth mbarrier; rows of 272 bytes (free of bank conflicts) for tr = 1, in 16-byte
   // pieces (256 bulk copies of a row took 10k cycles to issue)
@@ -263,10 +361,7 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
       cp_async_commit();
     } else if (uwarp == kIssueWarp) {
       asm volatile("fence.proxy.async;" ::: "memory");
-      if (lane == 0)
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(um.mbar + 24),
-                     "r"((uint32_t)((r1 - r0) * kb * 8))
-                     : "memory");
+      if (lane == 0) mbar_expect(um.mbar + 24, (r1 - r0) * kb * 8);
       __syncwarp();
       for (int a = lane; a < kb; a += 32)
         bulk_copy(sm + kDigRaw + (a * kDigRows + r0) * 8, X + r0 + (size_t)(c0 + a) * nb, (r1 - r0) * 8, um.mbar + 24);
@@ -274,7 +369,7 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
   };
   // waits until this thread's part of it is there (all of it for tr = 0)
   auto wait_v = [&]() {
-    if (tr) {
+    if (tr && !kPre) {
       cp_async_wait_all();
       return true;
     }
@@ -300,8 +395,13 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
       ct[k] = (top && lane < ncols && arow + k < kb) ? ldg(Cp + toff(c0 + arow + k, col0 + lane, nb, tr)) : 0.0;
   };
 
-  prefetch_v(blk_of(0) * ib);
-  load_t(blk_of(0) * ib);
+  if constexpr (kPre) {
+    if (uwarp == kIssueWarp) load_image(blk_of(0));
+    head = load_head(blk_of(0));
+  } else {
+    prefetch_v(blk_of(0) * ib);
+    load_t(blk_of(0) * ib);
+  }
   load_ct(blk_of(0) * ib);
 
   // ---- load the strip, find E_c -----------------------------------------------------------------
@@ -347,56 +447,69 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
     c0 = blk_of(bb) * ib;
     v0 = type == UNMQR ? c0 : 0;
     v1 = type == TTMQR ? c0 + kb : nb;
-    ok = wait_v() && ok;
-    if (tr) __syncthreads();
-    uint32_t hv = 0;                   // largest |v| (high word)
-    {
-      const bool vrow = r >= v0 && r < v1;
-#pragma unroll
-      for (int g = 0; g < 2; ++g) {
-        double x[8];
-        if (tr) {
-          const double2* p = reinterpret_cast<const double2*>(sm + kDigRaw + r * 272 + (cb + 8 * g) * 8);
-#pragma unroll
-          for (int a = 0; a < 4; ++a) {
-            const double2 d = p[a];
-            x[2 * a] = d.x;
-            x[2 * a + 1] = d.y;
-          }
-        } else {
-          const double* p = reinterpret_cast<const double*>(sm + kDigRaw) + (cb + 8 * g) * kDigRows + r;
-#pragma unroll
-          for (int a = 0; a < 8; ++a) x[a] = p[a * kDigRows];
-        }
-        const bool in = vrow && cb + 8 * g < kb;        // (kb is a multiple of 8)
-        const int d = r - (c0 + cb + 8 * g);            // 0 on the diagonal of column a = 0
-        if (type == UNMQR) {
-#pragma unroll
-          for (int a = 0; a < 8; ++a) x[a] = d > a ? x[a] : (d == a ? 1.0 : 0.0);
-        } else if (type == TTMQR) {
-#pragma unroll
-          for (int a = 0; a < 8; ++a) x[a] = d <= a ? x[a] : 0.0;
-        }
-        int64_t vf[8];
-#pragma unroll
-        for (int a = 0; a < 8; ++a) {
-          x[a] = in ? x[a] : 0.0;
-          hv = max(hv, (uint32_t)__double2hiint(x[a]) & 0x7fffffffu);
-          vf[a] = to_fixed(x[a], 62);
-        }
-        put_digits(sm + kDigV, r, 2 * ch + g, vf);
+    int eT;
+    if constexpr (kPre) {
+      if (!__syncthreads_and(ok ? 1 : 0)) {         // (also: the last block's products and scratch are done with)
+        ok = false;
+        break;
       }
-      uint32_t ht = max((uint32_t)__double2hiint(tv[0]) & 0x7fffffffu, (uint32_t)__double2hiint(tv[1]) & 0x7fffffffu);
-      ht = __reduce_max_sync(kFull, ht);
-      if (lane == 0) red[warp] = ht;
+      if (!head.x) {                                // uniform: the rest goes to the FP64 units
+        wait_v();
+        break;
+      }
+      eT = head.y;
+    } else {
+      ok = wait_v() && ok;
+      if (tr) __syncthreads();
+      uint32_t hv = 0;                   // largest |v| (high word)
+      {
+        const bool vrow = r >= v0 && r < v1;
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          double x[8];
+          if (tr) {
+            const double2* p = reinterpret_cast<const double2*>(sm + kDigRaw + r * 272 + (cb + 8 * g) * 8);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+              const double2 d = p[a];
+              x[2 * a] = d.x;
+              x[2 * a + 1] = d.y;
+            }
+          } else {
+            const double* p = reinterpret_cast<const double*>(sm + kDigRaw) + (cb + 8 * g) * kDigRows + r;
+#pragma unroll
+            for (int a = 0; a < 8; ++a) x[a] = p[a * kDigRows];
+          }
+          const bool in = vrow && cb + 8 * g < kb;        // (kb is a multiple of 8)
+          const int d = r - (c0 + cb + 8 * g);            // 0 on the diagonal of column a = 0
+          if (type == UNMQR) {
+#pragma unroll
+            for (int a = 0; a < 8; ++a) x[a] = d > a ? x[a] : (d == a ? 1.0 : 0.0);
+          } else if (type == TTMQR) {
+#pragma unroll
+            for (int a = 0; a < 8; ++a) x[a] = d <= a ? x[a] : 0.0;
+          }
+          int64_t vf[8];
+#pragma unroll
+          for (int a = 0; a < 8; ++a) {
+            x[a] = in ? x[a] : 0.0;
+            hv = max(hv, (uint32_t)__double2hiint(x[a]) & 0x7fffffffu);
+            vf[a] = to_fixed(x[a], 62);
+          }
+          put_digits(sm + kDigV, r, 2 * ch + g, vf);
+        }
+        uint32_t ht = max((uint32_t)__double2hiint(tv[0]) & 0x7fffffffu, (uint32_t)__double2hiint(tv[1]) & 0x7fffffffu);
+        ht = __reduce_max_sync(kFull, ht);
+        if (lane == 0) red[warp] = ht;
+      }
+      // the staged V is free from here on: the C digits take its place.  1: a wait ran out, 2: |v| > 1 (not finite)
+      if (__syncthreads_or(!ok || hv > 0x3ff00000u)) {
+        if (!__syncthreads_and(ok ? 1 : 0)) ok = false;
+        break;                           // uniform: the rest goes to the FP64 units
+      }
+      eT = max((int)(__reduce_max_sync(kFull, red[lane & 15]) >> 20) - 1022, 1);
+      if (eT > 12) break;
     }
-    // the staged V is free from here on: the C digits take its place.  1: a wait ran out, 2: |v| > 1 (not finite)
-    if (__syncthreads_or(!ok || hv > 0x3ff00000u)) {
-      if (!__syncthreads_and(ok ? 1 : 0)) ok = false;
-      break;                           // uniform: the rest goes to the FP64 units
-    }
-    const int eT = max((int)(__reduce_max_sync(kFull, red[lane & 15]) >> 20) - 1022, 1);
-    if (eT > 12) break;
     // ---- C digits ---------------------------------------------------------------------------------
 #pragma unroll
     for (int g = 0; g < 2; ++g) put_digits(sm + kDigC, r, 2 * ch + g, cf + 8 * g);
@@ -409,6 +522,7 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
       const uint32_t i0 = umma_idesc_f16(128, 32 * kDigN, true, true), i1 = umma_idesc_f16(128, 128, true, true);
       const int k0 = uniform(v0 >> 4), k1 = uniform((v1 + 15) >> 4);
       const uint64_t da = digit_desc(uV + k0 * 1024, kDigSlice), db = digit_desc(uC + k0 * 1024, kDigSlice);
+      if constexpr (kPre) ok = wait_v() && ok;
 #pragma unroll 4
       for (int k = 0; k < k1 - k0; ++k) {      // 16 rows: 1024 bytes
         umma_f16(utm, da + k * 64, db + k * 64, i0, k > 0);
@@ -416,7 +530,8 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
       }
       umma_commit_warp(um.mbar);
     }
-    ok = mbar_wait(um.mbar, um.phase & 1u, prm.wait_ns);
+    if (kPre && uwarp != kIssueWarp) um.phase ^= 8u;      // (that warp alone waits for V)
+    ok = mbar_wait(um.mbar, um.phase & 1u, prm.wait_ns) && ok;
     um.phase ^= 1u;
     __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -424,24 +539,35 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
     const double ctv[2] = {ct[0], ct[1]};
     const int h0 = v0 >> 7, h1 = (v1 + 127) >> 7;       // h0 .. h1 - 1: halves of 128 rows of this block
     int2* Ts = reinterpret_cast<int2*>(sm + kDigT);       // op(T)(a, t) at t 34 + a: 2^28 x + y = T 2^(56 - eT)
-    if (kb != 32) {
-      for (int o = tid; o < 1024; o += kThreads) Ts[(o >> 5) * 34 + (o & 31)] = make_int2(0, 0);
-      __syncthreads();
-    }
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int o = tid + k * kThreads, i = kb == 32 ? o & 31 : o % kb, j = kb == 32 ? o >> 5 : o / kb;
-      if (o < kb * kb) {
-        const int64_t f = to_fixed(tv[k], 63 - eT) >> 7;
-        const int h = (int)((f + (1 << 27)) >> 28), l = (int)(f - ((int64_t)h << 28));
-        Ts[notrans ? j * 34 + i : i * 34 + j] = make_int2(h, l);
+    if constexpr (kPre) {
+      if (uwarp == kIssueWarp && lane == 0) {
+        mbar_expect(um.mbar + 32, kDigTBytes);
+        bulk_copy(Ts, vd + (size_t)blk_of(bb) * digit_block_bytes(nb) + kDigN * img, kDigTBytes, um.mbar + 32);
       }
-    }
-    if (bb + 1 < nbk) {
-      const int cn = blk_of(bb + 1) * ib;
-      prefetch_v(cn);
-      load_t(cn);
-      load_ct(cn);
+      if (bb + 1 < nbk) {
+        head = load_head(blk_of(bb + 1));
+        load_ct(blk_of(bb + 1) * ib);
+      }
+    } else {
+      if (kb != 32) {
+        for (int o = tid; o < 1024; o += kThreads) Ts[(o >> 5) * 34 + (o & 31)] = make_int2(0, 0);
+        __syncthreads();
+      }
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int o = tid + k * kThreads, i = kb == 32 ? o & 31 : o % kb, j = kb == 32 ? o >> 5 : o / kb;
+        if (o < kb * kb) {
+          const int64_t f = to_fixed(tv[k], 63 - eT) >> 7;
+          const int h = (int)((f + (1 << 27)) >> 28), l = (int)(f - ((int64_t)h << 28));
+          Ts[notrans ? j * 34 + i : i * 34 + j] = make_int2(h, l);
+        }
+      }
+      if (bb + 1 < nbk) {
+        const int cn = blk_of(bb + 1) * ib;
+        prefetch_v(cn);
+        load_t(cn);
+        load_ct(cn);
+      }
     }
     // ---- partial sums of W 2^(62 - E_c): lane = (digit j = q of V, reflector), 8 columns per warp -------
     int64_t* P = reinterpret_cast<int64_t*>(sm + kDigP);
@@ -467,6 +593,10 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
     }
     __syncthreads();
     // ---- phase 2: W2 = op(T) W in integers, Ct -= W2, digits of W2 ----------------------------------
+    if constexpr (kPre) {
+      ok = mbar_wait(um.mbar + 32, (um.phase >> 4) & 1u, prm.wait_ns) && ok;
+      um.phase ^= 16u;
+    }
     int64_t w2[2];
     {
       int64_t A0 = 0, A1 = 0, B0 = 0, B1 = 0, D0 = 0, D1 = 0;
@@ -514,8 +644,14 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
       if (top && lane < ncols && arow + k < kb)
         stg(Cp + toff(c0 + arow + k, col0 + lane, nb, tr), from_fixed(c63[k] - 2 * w2[k], 63 - myE));
     // ---- C -= V W2 in integers: C 2^(63 - E_c) loses D_g 2^(51 - 8 g) -------------------------------
+    if (kPre && uwarp == kIssueWarp && bb + 1 < nbk) {
+      // V's place is free when the last half's products are (the first half's were issued before them)
+      ok = mbar_wait(um.mbar + 8 * h1, (um.phase >> h1) & 1u, prm.wait_ns) && ok;
+      __syncwarp();
+      load_image(blk_of(bb + 1));
+    }
     if (hw >= h0 && hw < h1) {         // warp-uniform
-      ok = mbar_wait(um.mbar + 8 + 8 * hw, (um.phase >> (1 + hw)) & 1u, prm.wait_ns);
+      ok = mbar_wait(um.mbar + 8 + 8 * hw, (um.phase >> (1 + hw)) & 1u, prm.wait_ns) && ok;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       __syncwarp();
 #pragma unroll
@@ -542,8 +678,8 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
   // in flight are waited for (with the same limit)
   if (!__syncthreads_and(ok ? 1 : 0)) {
     if (tid == 0) atomicCAS(prm.err, 0, DERR_TIMEOUT);
-    for (int b = 0; b < 4; ++b) mbar_wait(um.mbar + 8 * b, ((um.phase >> b) & 1u) ^ 1u, prm.wait_ns);
-    mbar_wait(um.mbar + 24, (um.phase >> 3) & 1u, prm.wait_ns);
+    for (int b = 0; b < 5; ++b) mbar_wait(um.mbar + 8 * b, ((um.phase >> b) & 1u) ^ 1u, prm.wait_ns);
+    for (int b = 3; b < 5; ++b) mbar_wait(um.mbar + 8 * b, (um.phase >> b) & 1u, prm.wait_ns);
     cp_async_wait_all();
     __syncthreads();
     return nbk;
