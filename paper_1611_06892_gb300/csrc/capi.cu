@@ -67,6 +67,8 @@ struct BatchPlan {
   int64_t tot0 = 0, tot1 = 0, totT = 0, totV = 0, tiles_all = 0, cols_all = 0;
   size_t smem = 0;
   bool digits = false;          // FP64: some matrix's updates run as digit products
+  int umma_cols = 0;            // FP32 storage: TMEM columns and shared memory of the updates on tcgen05
+  size_t smem_umma = 0;
   int ntasks = 0;
   PlanDev prog;                 // the merged device program
   void* d_mats = nullptr;       // info on the device
@@ -193,19 +195,17 @@ int run_exec(bidiag_handle h, const PlanDev& pd, int ntasks, void* b0, int64_t n
              int64_t n2, void* T, int npanels, int nb, int ib, int w, int esize, bool timed = false,
              const bd::MatInfo* d_mats = nullptr, int nmats = 0, size_t smem_batch = 0,
              const void* const* bx = nullptr, const int64_t* nx = nullptr, const bd::BwdParams* bwd = nullptr,
-             int auto_window = 0, bool digits_batch = false, int64_t vd_bytes = 0) {
+             int auto_window = 0, bool digits_batch = false, int64_t vd_bytes = 0,
+             int umma_batch = 0, size_t smem_umma = 0) {
   if (ntasks == 0) return BIDIAG_OK;
   size_t smem = d_mats ? smem_batch : (bwd ? bd::bwd_smem_bytes(nb, ib, bwd->hw, esize) : bd::exec_smem_bytes(nb, ib, w, esize));
-  // tcgen05 updates (FP32 forward, one CTA per SM): TMEM for one accumulator of N = max(w, ib) (rounded to
-  // 16) columns per 128-row chunk of the tile and per k-step of 8, allocated as a power of two of at
-  // least 32 columns, and the shared memory of that path's layout
+  // tcgen05 updates (FP32 forward, one CTA per SM): TMEM and the shared memory of that path's layout (a batch: the
+  // most any of its matrices wants)
   int umma_cols = 0;
-  if (esize == 4 && !bwd && !d_mats && h->f32_simt == 0 && nb % 16 == 0 && ib == 32 && w <= 64) {
-    const int need = ((nb + 127) / 128) * (ib / 8) * ((std::max(w, ib) + 15) / 16 * 16);
-    int cols = 32;
-    while (cols < need) cols *= 2;
-    const size_t su = std::max(smem, bd::umma_smem_bytes(nb, ib, w));
-    if (cols <= 512 && su <= h->smem_optin && bd::exec_set_smem(su, esize, false) == cudaSuccess &&
+  if (esize == 4 && !bwd && h->f32_simt == 0) {
+    const int cols = d_mats ? umma_batch : bd::umma_tmem(nb, ib, w);
+    const size_t su = std::max(smem, d_mats ? smem_umma : bd::umma_smem_bytes(nb, ib, w));
+    if (cols > 0 && su <= h->smem_optin && bd::exec_set_smem(su, esize, false) == cudaSuccess &&
         bd::exec_max_ctas_per_sm(su, esize, false) == 1) {
       umma_cols = cols;
       smem = su;
@@ -824,6 +824,10 @@ int band_batched_impl(bidiag_handle h, int64_t count, const int64_t* m, const in
     const BatchPlan::One& o = mats[(size_t)b];
     bp->smem = std::max(bp->smem, bd::exec_smem_bytes(o.nb, o.ib, o.w, esize));
     bp->digits = bp->digits || bd::digits_tmem(o.nb, o.ib, o.w) > 0;
+    if (const int cols = bd::umma_tmem(o.nb, o.ib, o.w)) {
+      bp->umma_cols = std::max(bp->umma_cols, cols);
+      bp->smem_umma = std::max(bp->smem_umma, bd::umma_smem_bytes(o.nb, o.ib, o.w));
+    }
   }
   // storage layout
   bp->info.resize((size_t)count);
@@ -831,14 +835,16 @@ int band_batched_impl(bidiag_handle h, int64_t count, const int64_t* m, const in
     const bd::Plan& pl = mats[(size_t)b].pd->plan;
     bd::MatInfo& mi = bp->info[(size_t)b];
     const int64_t t2 = (int64_t)pl.nb * pl.nb;
+    // (every matrix starts on a 16-byte boundary, whatever the tile sizes before it: bulk and 16-byte copies)
+    auto aligned = [](int64_t x) { return (x + 31) / 32 * 32; };
     mi.off[0] = bp->tot0;
     mi.ntiles[0] = (int64_t)pl.p * pl.q;
-    bp->tot0 += mi.ntiles[0] * t2;
+    bp->tot0 = aligned(bp->tot0 + mi.ntiles[0] * t2);
     mi.off[1] = bp->tot1;
     mi.ntiles[1] = pl.variant == BIDIAG_RBIDIAG ? (int64_t)pl.q * pl.q : 0;
-    bp->tot1 += mi.ntiles[1] * t2;
+    bp->tot1 = aligned(bp->tot1 + mi.ntiles[1] * t2);
     mi.offT = bp->totT;
-    bp->totT += (int64_t)std::max(1, pl.npanels) * pl.ib * pl.nb;
+    bp->totT = aligned(bp->totT + (int64_t)std::max(1, pl.npanels) * pl.ib * pl.nb);
     mi.nb = pl.nb;
     mi.ib = pl.ib;
     mi.w = pl.strip_w;
@@ -936,7 +942,7 @@ int band_batched_impl(bidiag_handle h, int64_t count, const int64_t* m, const in
   }
   rc = run_exec(h, bp->prog, bp->ntasks, store->tiles, tiles_all, store->tiles2, tot1 ? 1 : 0, nullptr, 0, store->T,
                 0, 0, 1, 1, esize, timed, static_cast<const bd::MatInfo*>(bp->d_mats), (int)count, smem, nullptr, nullptr,
-                nullptr, 0, bp->digits, bp->totV);
+                nullptr, 0, bp->digits, bp->totV, bp->umma_cols, bp->smem_umma);
   if (rc) return bail(rc);
   h->timed = timed;
   e = bd::launch_extract_batched(d_ex, (int)count, cols_all, esize, h->stream);

@@ -1033,14 +1033,21 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint3
 __host__ __device__ constexpr uint32_t umma_idesc_tf32(int m, int n) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
+// MMAs and their commit are issued by a whole warp, one elected lane (always the same) executing: with warp-uniform
+// operands the descriptors stay in uniform registers.  From a branch of one thread each MMA cost 143 - 202 cycles of
+// that thread's instructions whatever its size (M 128, N 224, K 16 takes the tensor pipe 112).
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(kFull, x, 0); }
 __device__ __forceinline__ void umma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
       "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
 __device__ __forceinline__ void umma_commit(uint32_t mbar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
+  asm volatile(
+      "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(mbar)
+      : "memory");
 }
 // Bounded wait for the mbarrier phase with the given parity; false if the limit ran out.
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, uint64_t limit_ns) {
@@ -1181,16 +1188,18 @@ __device__ bool apply_rm_umma(const float* Vh, const float* Vl, int vrows, int k
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const int nks = kb >> 3, mch = (vrows + 127) >> 7;
-  if (threadIdx.x == 0) {
+  if (uniform(threadIdx.x >> 5) == 0) {
     const uint32_t sbo = (uint32_t)(kb >> 2) * 128u, idesc = umma_idesc_tf32(128, npad);
-    const uint32_t vh = smem_u32(Vh), vl = smem_u32(Vl), bh = smem_u32(Bh), bl = smem_u32(Bl);
+    const uint64_t vh = umma_desc(uniform(smem_u32(Vh)), 128, sbo), vl = umma_desc(uniform(smem_u32(Vl)), 128, sbo);
+    const uint64_t bh = umma_desc(uniform(smem_u32(Bh)), 128, sbo), bl = umma_desc(uniform(smem_u32(Bl)), 128, sbo);
+    uint32_t d = uniform(um.tmem);
     for (int mc = 0; mc < mch; ++mc)
       for (int ks = 0; ks < nks; ++ks) {
-        const uint32_t d = um.tmem + (uint32_t)((mc * nks + ks) * npad);
-        const uint32_t ao = (uint32_t)mc * 16u * sbo + (uint32_t)ks * 256u, bo = (uint32_t)ks * 256u;
-        umma_tf32(d, umma_desc(vl + ao, 128, sbo), umma_desc(bh + bo, 128, sbo), idesc, 0);
-        umma_tf32(d, umma_desc(vh + ao, 128, sbo), umma_desc(bl + bo, 128, sbo), idesc, 1);
-        umma_tf32(d, umma_desc(vh + ao, 128, sbo), umma_desc(bh + bo, 128, sbo), idesc, 1);
+        const uint64_t ao = (uint64_t)mc * sbo + (uint64_t)ks * 16u, bo = (uint64_t)ks * 16u;   // in 16-byte units
+        umma_tf32(d, vl + ao, bh + bo, idesc, 0);
+        umma_tf32(d, vh + ao, bl + bo, idesc, 1);
+        umma_tf32(d, vh + ao, bh + bo, idesc, 1);
+        d += (uint32_t)npad;
       }
     umma_commit(um.mbar);
   }
@@ -1453,6 +1462,9 @@ __device__ bool task_update_umma(unsigned char* smb, int type, const float* X, f
   const int npad = (ncols + 15) & ~15;
   if (um.ncols_alloc == 0 || kb != 32 || (nb & 15) || (ncols & 31) || ncols > 64 || ncols > (w > ib ? w : ib) ||
       ((nb + 127) >> 7) * (kb >> 3) * npad > (int)um.ncols_alloc)
+    return false;
+  if ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Cp) | reinterpret_cast<uintptr_t>(C) |
+       reinterpret_cast<uintptr_t>(Tg)) & 15)
     return false;
   const UmmaLayout L = layout_umma(nb, ib, w);
   float* sm = reinterpret_cast<float*>(smb + kHeaderDoubles * sizeof(double));
@@ -2505,6 +2517,14 @@ cudaError_t extract_t(const E* tiles, int64_t rows_t, int nb, int64_t n, E* ab, 
 size_t exec_smem_bytes(int nb, int ib, int w, int esize) {
   const Layout a = layout_panel(nb, ib, esize), b = layout_update(nb, ib, w, esize);
   return kHeaderDoubles * sizeof(double) + (size_t)esize * (size_t)(a.total > b.total ? a.total : b.total);
+}
+
+int umma_tmem(int nb, int ib, int w) {
+  if (nb % 16 || ib != 32 || w > 64) return 0;
+  const int need = ((nb + 127) / 128) * (ib / 8) * (((w > ib ? w : ib) + 15) / 16 * 16);
+  int cols = 32;
+  while (cols < need) cols *= 2;
+  return cols <= 512 ? cols : 0;
 }
 
 size_t umma_smem_bytes(int nb, int ib, int w) {

@@ -88,6 +88,9 @@ struct ExecParams {
 
 // Shared memory (bytes) the executor needs for (nb, ib, w) and element size esize (8 or 4).
 size_t exec_smem_bytes(int nb, int ib, int w, int esize);
+// FP32 forward executor: TMEM columns its updates want on tcgen05, a power of two of at least 32 (0: the sizes do not
+// take that path): one accumulator of N = max(w, ib) (rounded to 16) columns per 128-row chunk and k-step of 8.
+int umma_tmem(int nb, int ib, int w);
 // Dynamic shared memory of the FP32 forward executor when its updates take the tcgen05 path (ib 32).
 size_t umma_smem_bytes(int nb, int ib, int w);
 // FP64 forward executor: TMEM columns its updates need to run as digit products on tcgen05 (0: the sizes stay on

@@ -125,6 +125,7 @@ __device__ __forceinline__ void inverse32(const double* G, const double* d, doub
 __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, double* X, double* A, int tr, double* Tg, int nb,
                                                int ib, int b, unsigned char* vd, Umma& um, const ExecParams& prm) {
   if ((smem_u32(sm) & 511) || (kind == PM_GE && (b + 1) * ib == nb)) return false;
+  if ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(A)) & 15) return false;      // 16-byte loads and stores
   int* colE = reinterpret_cast<int*>(sm + kDigHead);                     // E_c
   uint32_t* red = reinterpret_cast<uint32_t*>(sm + kDigHead + 128);      // reduction scratch of column_exponents, then:
   int64_t* dinv = reinterpret_cast<int64_t*>(red);                       //   1 / U_jj (2^57),
@@ -221,7 +222,7 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
           umma_f16(utm + 256, dr + (4 * 2048 >> 4) + k * 64, dr + k * 64, i1, 1);
         }
       }
-      umma_commit_warp(um.mbar);
+      umma_commit(um.mbar);
     }
     ok = mbar_wait(um.mbar, um.phase & 1u, prm.wait_ns) && ok;
     um.phase ^= 1u;
@@ -341,7 +342,7 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
         for (int ks = 0; ks < 2; ++ks)
           umma_f16(utm + 256 * h + 32 * j, da + ((j * kDigSlice + ks * 32) >> 4) + h * 512, db + ks * 16,
                    umma_idesc_f16(128, 32 * (8 - j), false, false), j + ks > 0);
-      umma_commit_warp(um.mbar + 8 + 8 * h);
+      umma_commit(um.mbar + 8 + 8 * h);
     }
   }
   if (hw >= h0 && hw < h1) {           // warp-uniform

@@ -56,20 +56,11 @@ __host__ __device__ constexpr uint32_t umma_idesc_f16(int m, int n, bool a_mn, b
   return (1u << 4) | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16) | ((uint32_t)(n >> 3) << 17) |
          ((uint32_t)(m >> 4) << 24);
 }
-// Issued by a whole warp, one elected lane (always the same) executing: with warp-uniform operands the descriptors
-// stay in uniform registers.  From a branch of one thread each MMA cost 145 - 200 cycles of that thread's
-// instructions, whatever its size.
 __device__ __forceinline__ void umma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n elect.sync _|e, 0xffffffff;\n"
       " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
       "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-__device__ __forceinline__ void umma_commit_warp(uint32_t mbar) {
-  asm volatile(
-      "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
-      " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(mbar)
-      : "memory");
 }
 // size bytes (a multiple of 16) from global to shared memory, both 16-byte aligned
 __device__ __forceinline__ void bulk_copy(void* dst, const void* src, int size, uint32_t mbar) {
@@ -81,7 +72,6 @@ __device__ __forceinline__ void mbar_expect(uint32_t mbar, int bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
 }
 constexpr int kIssueWarp = 12;       // of the second row half: the first half's warps go on during the MMAs
-__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(kFull, x, 0); }
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* r) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
@@ -319,7 +309,8 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
                                                int blk1, int col0, int ncols, const unsigned char* vd, Umma& um,
                                                const ExecParams& prm) {
   static_assert(kThreads == 512, "two threads a row");
-  if (smem_u32(sm) & 511) return 0;                                      // the swizzle's alignment
+  if (smem_u32(sm) & 511) return 0;                                      // the swizzle's alignment, and the copies'
+  if ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Cp) | reinterpret_cast<uintptr_t>(C)) & 15) return 0;
   int* colE = reinterpret_cast<int*>(sm + kDigHead);                     // E_c
   uint32_t* red = reinterpret_cast<uint32_t*>(sm + kDigHead + 128);      // 16 x 16 reduction scratch
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -528,7 +519,7 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
         umma_f16(utm, da + k * 64, db + k * 64, i0, k > 0);
         umma_f16(utm + 256, da + (4 * kDigSlice >> 4) + k * 64, db + k * 64, i1, k > 0);
       }
-      umma_commit_warp(um.mbar);
+      umma_commit(um.mbar);
     }
     if (kPre && uwarp != kIssueWarp) um.phase ^= 8u;      // (that warp alone waits for V)
     ok = mbar_wait(um.mbar, um.phase & 1u, prm.wait_ns) && ok;
@@ -636,7 +627,7 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
           for (int ks = 0; ks < 2; ++ks)
             umma_f16(utm + 256 * h + 32 * j, da + ((j * kDigSlice + ks * 32) >> 4) + h * 512, db + ks * 16,
                      umma_idesc_f16(128, 32 * (8 - j), false, false), j + ks > 0);
-        umma_commit_warp(um.mbar + 8 + 8 * h);
+        umma_commit(um.mbar + 8 + 8 * h);
       }
     }
 #pragma unroll

@@ -80,3 +80,19 @@ def test_values_out_of_range_take_the_fp64_units(handle, bad):
     ref = OB.bidiag_band(A, 96, 32, T.GREEDY, T.BIDIAG)
     ab = band(handle, A, 96, 32, "greedy", "bidiag").band().cpu().numpy()
     assert np.abs(ab - ref["ab"]).max() <= TOL * np.linalg.norm(A)
+
+
+@pytest.mark.parametrize("dtype", ["float64", "float32"])
+def test_batch_with_odd_tiles_beside(handle, dtype):
+    """Tiles whose sizes leave the next matrix's storage unaligned (nb 7, 9, 33) beside ones that take the tensor-core
+    paths: each result is bitwise that of the matrix alone."""
+    import torch
+    cfg = [(7, 7), (96, 32), (9, 3), (64, 32), (33, 11), (128, 32), (64, 16)]
+    As = [torch.from_numpy(np.asfortranarray(inputs.gaussian(90 + 41 * i, 61 + 29 * i, seed=i)).astype(dtype, order="F")).cuda()
+          for i in range(len(cfg))]
+    res = handle.band_batched(As, [c[0] for c in cfg], [c[1] for c in cfg], ["greedy"] * 7, ["bidiag"] * 7)
+    handle.sync()
+    for A, (nb, ib), r in zip(As, cfg, res):
+        single = handle.band(A, nb, ib, "greedy", "bidiag")
+        handle.sync()
+        assert torch.equal(r.band(), single.band()), (nb, ib)
