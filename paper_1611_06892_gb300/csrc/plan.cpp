@@ -21,6 +21,7 @@
 #include <deque>
 #include <functional>
 #include <map>
+#include <queue>
 #include <stdexcept>
 
 namespace bd {
@@ -424,8 +425,8 @@ int best_split(int p, int q, int tree, int64_t R, int64_t* cp) {
 // tile (a diagonal block is split into its strict upper part, diagonal and strict lower part) and per
 // T block: read-after-write, write-after-write and write-after-read.  An update strip depends on the
 // last sub-task of its panel task for the reflectors it applies (the panel's sub-tasks are chained, and
-// a factored region is never written again).  Sub-tasks are queued by decreasing bottom level (longest
-// weighted path to the end), a topological order since every weight is positive.
+// a factored region is never written again).  Sub-tasks are queued in the order of a list schedule by
+// bottom level (longest weighted path to the end), see list_schedule.
 // ---------------------------------------------------------------------------------------------
 namespace {
 
@@ -507,17 +508,73 @@ inline int32_t make_op(int type, bool tr, bool notrans, int strip, int blk, int 
 
 }  // namespace
 
-// Priority weight of a sub-task: its Table 1 flops times the time per flop of its kind relative to a
-// TSMQR strip, in percent (mode 1), measured from per-sub-task traces of the executor on a GB300 (nb 256,
-// ib 32; FP32 storage at 8192^2 with the tcgen05 updates, FP64 at 4096^2).  Mode 0 is the flop count
-// alone, with FP32-storage panel factors counted twice.
+// Modelled time of a sub-task in units of 10 ns, dispatch (1 us) included (mode 1), from per-sub-task traces of
+// the executor on a GB300 (ib 32).  rows: rows of V; blocks: panel blocks an update strip applies.
+//  * FP64 digit products (nb 256, 192 and 128): factors and panel-block updates take the same time whatever the
+//    rows (their cost is per column), strips a fixed time per block.
+//  * FP32 storage (nb 256 and 128, tcgen05 updates): factors and panel-block updates affine in the rows, strips in
+//    the flops.
+//  * FP64 on the FMA units: Table 1 flops, times the time per flop of the kind relative to a TSMQR strip.
+// Mode 0 is the flop count alone, with FP32-storage panel factors counted twice.
 enum WeightClass { W_PF_GE, W_PF_TS, W_PF_TT, W_PU_GE, W_PU_TS, W_PU_TT, W_UNMQR, W_TSMQR, W_TTMQR };
-static int64_t prio_weight(int64_t flops, int cls, int esize, int mode, bool digits) {
-  static const int64_t kF32[9] = {640, 400, 650, 125, 115, 210, 135, 100, 150};
+static int64_t sub_time(int64_t flops, int cls, int64_t rows, int ib, int blocks, int esize, int mode, bool digits) {
+  static const int64_t kDig[9] = {7700, 6200, 5800, 2250, 2500, 2100, 1180, 1380, 1220};
   static const int64_t kF64[9] = {71, 51, 74, 71, 70, 79, 117, 100, 119};
-  static const int64_t kDig[9] = {277, 124, 205, 183, 115, 171, 174, 100, 183};   // FP64, digit products (8192^2)
+  static const int64_t kF32Base[6] = {4000, 3700, 4500, 500, 600, 550}, kF32Row[6] = {17, 12, 14, 2, 2, 2};
+  static const int64_t kF32[3] = {576, 453, 650};   // per Mflop
+  constexpr int64_t kDispatch = 100;
   if (mode == 0) return (cls <= W_PF_TT && esize == 4 ? 2 : 1) * flops;
-  return std::max<int64_t>(1, flops * (esize == 4 ? kF32[cls] : (digits ? kDig[cls] : kF64[cls])) / 100);
+  if (digits) return kDispatch + kDig[cls] * (cls >= W_UNMQR ? blocks : 1);
+  if (esize == 8) return kDispatch + flops * kF64[cls] / 7300;
+  if (cls < W_UNMQR) return kDispatch + (kF32Base[cls] + kF32Row[cls] * rows) * ib / 32;
+  return kDispatch + 1400 + flops * kF32[cls - W_UNMQR] / 1000000;
+}
+
+// Queue order: the order in which a list schedule on the chip's SMs starts the sub-tasks (of the ready ones the one
+// with the longest weighted path to the end first), by the modelled times.  CTAs take the queue strictly in order, so
+// a queue sorted by that path alone let them wait on sub-tasks of the chain while ready strips stood behind them
+// (GB300, that order against this one: 8192^2 FP64 181.1 -> 170.0 ms, FP32 96.3 -> 89.4, 4096^2 45.1 -> 42.4, a batch
+// of 64 to 1024 columns FP64 15.4 -> 11.7, FP32 8.5 -> 8.0; scanning ahead of the head instead costs more than it
+// finds, 8192^2 186 ms with 1024 entries).  A sub-task is started after the ones it depends on: the order
+// is topological.  Sub-tasks are numbered topologically on input.
+static std::vector<int32_t> list_schedule(const std::vector<int64_t>& time, const std::vector<int64_t>& bottom,
+                                          const std::vector<int64_t>& dep_begin, const std::vector<int32_t>& deps) {
+  constexpr int kWorkers = 152;
+  const int32_t n = (int32_t)time.size();
+  std::vector<int64_t> first(n + 1, 0);
+  std::vector<int32_t> succ(deps.size()), open(n), order;
+  for (int32_t d : deps) ++first[d + 1];
+  for (int32_t y = 0; y < n; ++y) first[y + 1] += first[y];
+  {
+    std::vector<int64_t> at(first.begin(), first.end() - 1);
+    for (int32_t y = 0; y < n; ++y) {
+      open[y] = (int32_t)(dep_begin[y + 1] - dep_begin[y]);
+      for (int64_t d = dep_begin[y]; d < dep_begin[y + 1]; ++d) succ[at[deps[d]]++] = y;
+    }
+  }
+  using Item = std::pair<int64_t, int32_t>;
+  std::priority_queue<Item> ready;                                               // (bottom level, -number)
+  std::priority_queue<Item, std::vector<Item>, std::greater<Item>> running;      // (end, number)
+  for (int32_t y = 0; y < n; ++y)
+    if (open[y] == 0) ready.push({bottom[y], -y});
+  order.reserve(n);
+  int64_t now = 0;
+  for (int idle = kWorkers;;) {
+    for (; idle > 0 && !ready.empty(); --idle) {
+      const int32_t y = -ready.top().second;
+      ready.pop();
+      order.push_back(y);
+      running.push({now + time[y], y});
+    }
+    if (running.empty()) break;
+    for (now = running.top().first; !running.empty() && running.top().first == now; ++idle) {
+      const int32_t y = running.top().second;
+      running.pop();
+      for (int64_t e = first[y]; e < first[y + 1]; ++e)
+        if (--open[succ[e]] == 0) ready.push({bottom[succ[e]], -succ[e]});
+    }
+  }
+  return order;
 }
 
 void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int variant, int64_t R, int strip_w,
@@ -613,7 +670,7 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
         wr.push_back(it.t(slot, b));
         const int64_t rows = kind == PK_GE ? nb - (int64_t)b * ib : (kind == PK_TS ? nb : (int64_t)(b + 1) * ib);
         d.op = make_op(PF, lq, false, 0, b, kind);
-        last = g.add(d, prio_weight(12 * ib2 * rows, W_PF_GE + kind, esize, prio, digits), rd, wr, -1);
+        last = g.add(d, sub_time(12 * ib2 * rows, W_PF_GE + kind, rows, ib, 1, esize, prio, digits), rd, wr, -1);
         // PU(b, s)
         for (int s = b + 1; s < nblk; ++s) {
           rd.clear();
@@ -634,7 +691,7 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
           }
           rd.push_back(it.t(slot, b));
           d.op = make_op(PU, lq, false, s, b, kind);
-          last = g.add(d, prio_weight(6 * ib2 * rows, W_PU_GE + kind, esize, prio, digits), rd, wr, -1);
+          last = g.add(d, sub_time(6 * ib2 * rows, W_PU_GE + kind, rows, ib, 1, esize, prio, digits), rd, wr, -1);
         }
       }
       panel_last[x] = last;
@@ -659,7 +716,8 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
           }
         }
         d.op = make_op(t.type, lq, false, s, 0, 0);
-        g.add(d, prio_weight(per_strip, t.type == UNMQR ? W_UNMQR : (t.type == TSMQR ? W_TSMQR : W_TTMQR), esize, prio, digits),
+        g.add(d, sub_time(per_strip, t.type == UNMQR ? W_UNMQR : (t.type == TSMQR ? W_TSMQR : W_TTMQR), nb, ib, nblk,
+                          esize, prio, digits),
               rd, wr, panel_last[owner]);
       }
     } else {   // COPY(i, j): R part of A's tile (i, j) into the second phase's tile (i, j)
@@ -681,7 +739,7 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
           else if (br == bc) src.up(rd, br);
         }
       }
-      g.add(d, (int64_t)nb * nb, rd, wr, -1);
+      g.add(d, prio ? 100 + (int64_t)nb * nb / 10 : (int64_t)nb * nb, rd, wr, -1);   // 64 us at nb 256
     }
   }
 
@@ -692,16 +750,22 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
     bottom[y] += g.weight[y];
     for (int32_t dd : g.deps[y]) bottom[dd] = std::max(bottom[dd], bottom[y]);
   }
-  std::vector<int32_t> order(nsub);
-  for (int32_t y = 0; y < nsub; ++y) order[y] = y;
-  std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return bottom[a] > bottom[b]; });
+  std::vector<int64_t> dep_begin(nsub + 1, 0);
+  std::vector<int32_t> deps;
+  for (int32_t y = 0; y < nsub; ++y) {
+    deps.insert(deps.end(), g.deps[y].begin(), g.deps[y].end());
+    dep_begin[y + 1] = (int64_t)deps.size();
+  }
+  const std::vector<int32_t> order = list_schedule(g.weight, bottom, dep_begin, deps);
   std::vector<int32_t> pos(nsub);
   for (int32_t y = 0; y < nsub; ++y) pos[order[y]] = y;
   pl.dev.resize(nsub);
   pl.deps.clear();
   pl.prio.resize(nsub);
+  pl.time.resize(nsub);
   for (int32_t y = 0; y < nsub; ++y) {
     pl.prio[y] = bottom[order[y]];
+    pl.time[y] = g.weight[order[y]];
     DevTask e = g.sub[order[y]];
     e.dep_begin = (int32_t)pl.deps.size();
     for (int32_t dd : g.deps[order[y]]) {
@@ -1000,47 +1064,36 @@ void build_backward(const Plan& pl, BwdPlan& bp, bool split_strips) {
 void merge_programs(const std::vector<const Plan*>& plans, std::vector<DevTask>* dev, std::vector<int32_t>* deps) {
   const size_t np = plans.size();
   if (np >= (1u << 23)) throw std::invalid_argument("too many matrices in a batch");
-  size_t total = 0;
-  for (const Plan* pl : plans) total += pl->dev.size();
-  std::vector<size_t> head(np, 0);
-  std::vector<std::vector<int32_t>> gpos(np);
-  for (size_t b = 0; b < np; ++b) gpos[b].resize(plans[b]->dev.size());
-  // k-way merge by decreasing priority (ties: lower matrix index first)
-  using Item = std::pair<int64_t, int64_t>;   // (-prio, b)
-  std::vector<Item> heap;
-  auto push = [&](size_t b) {
-    if (head[b] < plans[b]->dev.size()) {
-      heap.push_back({-plans[b]->prio[head[b]], (int64_t)b});
-      std::push_heap(heap.begin(), heap.end(), std::greater<Item>());
+  // one program of all sub-tasks, matrix after matrix, then its list schedule
+  std::vector<int64_t> time, bottom, dep_begin{0};
+  std::vector<int32_t> gdeps, first{0}, mat;
+  for (size_t b = 0; b < np; ++b) {
+    const Plan& pl = *plans[b];
+    time.insert(time.end(), pl.time.begin(), pl.time.end());
+    bottom.insert(bottom.end(), pl.prio.begin(), pl.prio.end());
+    mat.insert(mat.end(), pl.dev.size(), (int32_t)b);
+    for (const DevTask& e : pl.dev) {
+      for (int32_t d = e.dep_begin; d < e.dep_end; ++d) gdeps.push_back(first[b] + pl.deps[d]);
+      dep_begin.push_back((int64_t)gdeps.size());
     }
-  };
-  for (size_t b = 0; b < np; ++b) push(b);
-  dev->clear();
-  dev->reserve(total);
-  std::vector<std::pair<int32_t, int32_t>> src;   // (matrix, local queue position) per global position
-  src.reserve(total);
-  while (!heap.empty()) {
-    std::pop_heap(heap.begin(), heap.end(), std::greater<Item>());
-    const size_t b = (size_t)heap.back().second;
-    heap.pop_back();
-    const int32_t y = (int32_t)head[b]++;
-    gpos[b][y] = (int32_t)src.size();
-    src.push_back({(int32_t)b, y});
-    push(b);
+    first.push_back((int32_t)time.size());
   }
+  const std::vector<int32_t> order = list_schedule(time, bottom, dep_begin, gdeps);
+  std::vector<int32_t> pos(order.size());
+  for (size_t g = 0; g < order.size(); ++g) pos[order[g]] = (int32_t)g;
+  dev->clear();
+  dev->reserve(order.size());
   deps->clear();
-  for (size_t g = 0; g < src.size(); ++g) {
-    const Plan* pl = plans[src[g].first];
-    DevTask e = pl->dev[src[g].second];
-    const int32_t b0 = e.dep_begin, b1 = e.dep_end;
+  for (size_t g = 0; g < order.size(); ++g) {
+    const int32_t y = order[g], b = mat[y];
+    DevTask e = plans[b]->dev[y - first[b]];
     e.dep_begin = (int32_t)deps->size();
-    for (int32_t d = b0; d < b1; ++d) {
-      const int32_t gd = gpos[src[g].first][pl->deps[d]];
-      if (gd >= (int32_t)g) throw std::logic_error("merged order is not topological");
-      deps->push_back(gd);
+    for (int64_t d = dep_begin[y]; d < dep_begin[y + 1]; ++d) {
+      if (pos[gdeps[d]] >= (int32_t)g) throw std::logic_error("merged order is not topological");
+      deps->push_back(pos[gdeps[d]]);
     }
     e.dep_end = (int32_t)deps->size();
-    e.flags = (e.flags & 0xff) | (src[g].first << 8);
+    e.flags = (e.flags & 0xff) | (b << 8);
     dev->push_back(e);
   }
 }

@@ -92,7 +92,8 @@ struct Plan {
   // device program
   std::vector<DevTask> dev;        // in queue (priority) order
   std::vector<int32_t> deps;       // indices into dev (queue positions)
-  std::vector<int64_t> prio;       // bottom level of each queued sub-task (flop-proportional weights)
+  std::vector<int64_t> prio;       // bottom level of each queued sub-task (modelled times)
+  std::vector<int64_t> time;       // modelled time of each
 };
 
 // Adjoint program of a plan (the reverse sweep).  Sub-task y of the forward program becomes its
@@ -134,13 +135,12 @@ int choose_variant(int p, int q, int tree, int64_t resources, int64_t* cp_bidiag
 int best_split(int p, int q, int tree, int64_t resources, int64_t* cp);
 // Full plan for a reduction: tasks, DAG, device sub-tasks ordered by critical-path priority.  esize
 // (8: FP64, 4: FP32 storage) and prio (1: calibrated per-kind times, 0: flop counts) only set the
-// priority weights.
+// modelled times.
 void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int variant, int64_t resources,
                 int strip_w, int esize = 8, int prio = 1);
 
-// Several independent plans as one device program: the queues are merged by decreasing bottom level
-// (each plan's own order is kept, so the result is topological), matrix b's sub-tasks carry b in
-// flags bits 8-31 and their dependencies are renumbered to the merged queue.
+// Several independent plans as one device program, in the order of one list schedule of all of them: matrix b's
+// sub-tasks carry b in flags bits 8-31 and their dependencies are renumbered to the merged queue.
 void merge_programs(const std::vector<const Plan*>& plans, std::vector<DevTask>* dev, std::vector<int32_t>* deps);
 
 // Tile size, inner blocking, tree and variant for one m x n matrix of a batch (the batched form's

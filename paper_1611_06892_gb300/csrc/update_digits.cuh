@@ -309,7 +309,7 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
                                                int blk1, int col0, int ncols, const unsigned char* vd, Umma& um,
                                                const ExecParams& prm) {
   static_assert(kThreads == 512, "two threads a row");
-  if (smem_u32(sm) & 511) return 0;                                      // the swizzle's alignment, and the copies'
+  if (smem_u32(sm) & 511) return 0;                                      // the swizzle's alignment, and the copies
   if ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Cp) | reinterpret_cast<uintptr_t>(C)) & 15) return 0;
   int* colE = reinterpret_cast<int*>(sm + kDigHead);                     // E_c
   uint32_t* red = reinterpret_cast<uint32_t*>(sm + kDigHead + 128);      // 16 x 16 reduction scratch
