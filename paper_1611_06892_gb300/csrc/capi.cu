@@ -111,7 +111,7 @@ struct bidiag_ctx {
   int tracing = 0;
   int f32_simt = 0;                // FP32 storage: updates by FFMA instead of 3xTF32 tensor-core products
   int f32_scalars64 = 0;           // FP32 storage: reflector scalars in FP64 instead of float pairs
-  int window = -1;                 // executor look-ahead (queue entries scanned); -1: by precision and variant
+  int window = -1;                 // executor look-ahead (queue entries scanned); -1: none, strict queue order
   int prio = 1;                    // priority weights of the device program: 1 calibrated per kind, 0 flops
   unsigned char* d_vd = nullptr;   // storage of published panel blocks kept between launches, and its bytes
   int64_t vd_cap = 0;
@@ -195,7 +195,7 @@ int run_exec(bidiag_handle h, const PlanDev& pd, int ntasks, void* b0, int64_t n
              int64_t n2, void* T, int npanels, int nb, int ib, int w, int esize, bool timed = false,
              const bd::MatInfo* d_mats = nullptr, int nmats = 0, size_t smem_batch = 0,
              const void* const* bx = nullptr, const int64_t* nx = nullptr, const bd::BwdParams* bwd = nullptr,
-             int auto_window = 0, bool digits_batch = false, int64_t vd_bytes = 0,
+             bool digits_batch = false, int64_t vd_bytes = 0,
              int umma_batch = 0, size_t smem_umma = 0) {
   if (ntasks == 0) return BIDIAG_OK;
   size_t smem = d_mats ? smem_batch : (bwd ? bd::bwd_smem_bytes(nb, ib, bwd->hw, esize) : bd::exec_smem_bytes(nb, ib, w, esize));
@@ -248,7 +248,7 @@ int run_exec(bidiag_handle h, const PlanDev& pd, int ntasks, void* b0, int64_t n
   prm.esize = esize;
   prm.f32_simt = h->f32_simt;
   prm.f32_scalars64 = h->f32_scalars64;
-  prm.window = h->window >= 0 ? h->window : auto_window;
+  prm.window = std::max(h->window, 0);
   prm.umma_cols = umma_cols;
   prm.mats = d_mats;
   prm.nmats = nmats;
@@ -561,8 +561,7 @@ int band_impl(bidiag_handle h, int64_t m, int64_t n, const E* d_A, int64_t lda, 
   rc = run_exec(h, *pd, (int)pd->plan.dev.size(), r->tiles, (int64_t)r->p * r->q, r->tiles2,
                 r->tiles2 ? (int64_t)r->q * r->q : 0, nullptr, 0, r->T, pd->plan.npanels, nb, ib, w, (int)sizeof(E),
                 timed, nullptr, 0, 0, nullptr, nullptr, nullptr,
-                (sizeof(E) == 8 && !r->tiles2 && !bd::digits_fit(nb, ib, w)) ? bd::kWindowF64BiDiag : 0, false,
-                (int64_t)pd->plan.npanels * (nb / ib) * bd::digit_block_bytes(nb));
+                false, (int64_t)pd->plan.npanels * (nb / ib) * bd::digit_block_bytes(nb));
   h->timed = timed;
   if (rc) return bail(rc);
   if (tiles2 && variant != BIDIAG_RBIDIAG) {
@@ -942,7 +941,7 @@ int band_batched_impl(bidiag_handle h, int64_t count, const int64_t* m, const in
   }
   rc = run_exec(h, bp->prog, bp->ntasks, store->tiles, tiles_all, store->tiles2, tot1 ? 1 : 0, nullptr, 0, store->T,
                 0, 0, 1, 1, esize, timed, static_cast<const bd::MatInfo*>(bp->d_mats), (int)count, smem, nullptr, nullptr,
-                nullptr, 0, bp->digits, bp->totV, bp->umma_cols, bp->smem_umma);
+                nullptr, bp->digits, bp->totV, bp->umma_cols, bp->smem_umma);
   if (rc) return bail(rc);
   h->timed = timed;
   e = bd::launch_extract_batched(d_ex, (int)count, cols_all, esize, h->stream);

@@ -51,12 +51,6 @@ struct BwdParams {
   int pu_split;             // column pieces of a panel-block update adjoint (1 or 2)
 };
 
-// Executor look-ahead of one-matrix FP64 BiDiag reductions (queue entries scanned for a ready sub-task):
-// 8192^2 1374 -> 1330 ms, 4096^2 232 -> 222 ms against strict queue order with sub-tasks on the FP64 units; FP32
-// storage, R-BiDiag, batches and the ten times shorter sub-tasks of the digit products (8192^2 196.6 ms in strict
-// order, 203.1 with the window) were not faster with it and keep strict order.
-constexpr int kWindowF64BiDiag = 1024;
-
 struct ExecParams {
   const DevTask* tasks;
   const int32_t* deps;
@@ -80,7 +74,10 @@ struct ExecParams {
                         // 1 = updates by FP32 FFMA, 2 = three-TF32 updates on the warp-level MMA only
   int umma_cols;        // forward programs: TMEM columns each CTA allocates for the tcgen05 phases (0: none)
   int f32_scalars64;    // FP32 tiles only: 1 = reflector beta / tau / scale in FP64 instead of float pairs
-  int window;           // queue entries from the head a CTA scans for a ready sub-task (0: strict queue order)
+  // queue entries from the head a CTA scans for a ready sub-task (0, the default: strict queue order; with the queue in
+  // the order of a list schedule scanning only costs: 8192^2 FP64 170 ms against 186 with 1024 entries, 4096^2 with tiles
+  // of 64 and ib 8 on the FMA units 504 against 582)
+  int window;
   unsigned char* vd;    // FP64 reductions with digit products: published panel blocks (digit_block_bytes each, by T slot
                         // and inner block; null: the updates make the digits of V themselves)
   BwdParams bwd;        // adjoint program only

@@ -178,7 +178,7 @@ extern "C" int bidiag_band_noalloc(int64_t m, int64_t n, const double* d_A, int6
     const char* wl = std::getenv("BIDIAG_WAIT_LIMIT_NS");
     prm.wait_ns = wl ? std::strtoull(wl, nullptr, 10) : 20000000000ull;
     prm.esize = 8;
-    prm.window = (tiles2 || bd::digits_fit(nb, ib, w)) ? 0 : bd::kWindowF64BiDiag;
+    prm.window = 0;
     if (bd::digits_tmem(nb, ib, w) > 0) {   // digit products on tcgen05, as bidiag_band runs them
       const size_t su = std::max(smem, bd::digits_smem_bytes());
       if (su <= (size_t)optin - 64 && bd::exec_set_smem(su, 8, false, true) == cudaSuccess &&

@@ -17,6 +17,7 @@
 #include "plan.h"
 
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <deque>
 #include <functional>
@@ -508,26 +509,62 @@ inline int32_t make_op(int type, bool tr, bool notrans, int strip, int blk, int 
 
 }  // namespace
 
+// Measured mean sub-task times of the executor, per storage precision and (nb, ib): see
+// autotune_table.inc for the command that writes them.  Classes: PF GE / TS / TT, PU GE / TS / TT,
+// UNMQR / TSMQR / TTMQR update strips.
+struct AutotuneRow {
+  int esize, nb, ib;
+  double us[9];
+};
+const AutotuneRow kAutotuneTable[] = {
+#include "autotune_table.inc"
+    {0, 0, 0, {0, 0, 0, 0, 0, 0, 0, 0, 0}},   // end marker
+};
+
 // Modelled time of a sub-task in units of 10 ns, dispatch (1 us) included (mode 1), from per-sub-task traces of
-// the executor on a GB300 (ib 32).  rows: rows of V; blocks: panel blocks an update strip applies.
+// the executor on a GB300.  rows: rows of V; blocks: panel blocks an update strip applies.
 //  * FP64 digit products (nb 256, 192 and 128): factors and panel-block updates take the same time whatever the
 //    rows (their cost is per column), strips a fixed time per block.
-//  * FP32 storage (nb 256 and 128, tcgen05 updates): factors and panel-block updates affine in the rows, strips in
-//    the flops.
-//  * FP64 on the FMA units: Table 1 flops, times the time per flop of the kind relative to a TSMQR strip.
+//  * FP32 storage with tcgen05 updates (ib 32, nb 256 and 128): factors and panel-block updates affine in the rows,
+//    strips in the flops.
+//  * Else the autotuner's table (strips of 32 columns) at the nearest tile size, in proportion to the flops (factors:
+//    to ib).
 // Mode 0 is the flop count alone, with FP32-storage panel factors counted twice.
 enum WeightClass { W_PF_GE, W_PF_TS, W_PF_TT, W_PU_GE, W_PU_TS, W_PU_TT, W_UNMQR, W_TSMQR, W_TTMQR };
-static int64_t sub_time(int64_t flops, int cls, int64_t rows, int ib, int blocks, int esize, int mode, bool digits) {
-  static const int64_t kDig[9] = {7700, 6200, 5800, 2250, 2500, 2100, 1180, 1380, 1220};
-  static const int64_t kF64[9] = {71, 51, 74, 71, 70, 79, 117, 100, 119};
+static int64_t sub_time(int64_t flops, int cls, int64_t rows, int nb, int ib, int esize, int mode, bool digits) {
+  static const int64_t kDig[9] = {6700, 5900, 5500, 2250, 2500, 2100, 1180, 1380, 1220};
   static const int64_t kF32Base[6] = {4000, 3700, 4500, 500, 600, 550}, kF32Row[6] = {17, 12, 14, 2, 2, 2};
   static const int64_t kF32[3] = {576, 453, 650};   // per Mflop
   constexpr int64_t kDispatch = 100;
   if (mode == 0) return (cls <= W_PF_TT && esize == 4 ? 2 : 1) * flops;
-  if (digits) return kDispatch + kDig[cls] * (cls >= W_UNMQR ? blocks : 1);
-  if (esize == 8) return kDispatch + flops * kF64[cls] / 7300;
-  if (cls < W_UNMQR) return kDispatch + (kF32Base[cls] + kF32Row[cls] * rows) * ib / 32;
-  return kDispatch + 1400 + flops * kF32[cls - W_UNMQR] / 1000000;
+  if (digits) return kDispatch + kDig[cls] * (cls >= W_UNMQR ? nb / ib : 1);
+  if (esize == 4 && ib == 32 && nb >= 96) {
+    if (cls < W_UNMQR) return kDispatch + kF32Base[cls] + kF32Row[cls] * rows;
+    return kDispatch + 1400 + flops * kF32[cls - W_UNMQR] / 1000000;
+  }
+  const AutotuneRow* best = nullptr;
+  double dist = 0.0;
+  for (const AutotuneRow* r = kAutotuneTable; r->esize; ++r) {
+    const double d = std::fabs(std::log2((double)nb / r->nb)) + std::fabs(std::log2((double)ib / r->ib));
+    if (r->esize == esize && (!best || d < dist)) {
+      best = r;
+      dist = d;
+    }
+  }
+  double us = best->us[cls];
+  if (cls <= W_PF_TT) {
+    us *= (double)ib / best->ib;
+  } else {
+    const double n = best->nb, k = best->ib;
+    const double ref = cls <= W_PU_TT ? (cls == W_PU_TS ? 6 : 3) * k * k * n : (cls == W_TSMQR ? 4 : 2) * n * n * 32;
+    double ratio = (double)flops / ref;
+    if (esize == 4 && cls >= W_UNMQR) {      // of a strip of FP32 storage 0.6 do not depend on its width
+      const double tile = (double)nb * nb / (n * n);
+      ratio = 0.6 * tile + 0.4 * ratio;
+    }
+    us = (us > 0.0 ? us : 10.0) * ratio;
+  }
+  return kDispatch + (int64_t)(100.0 * us);
 }
 
 // Queue order: the order in which a list schedule on the chip's SMs starts the sub-tasks (of the ready ones the one
@@ -535,8 +572,10 @@ static int64_t sub_time(int64_t flops, int cls, int64_t rows, int ib, int blocks
 // a queue sorted by that path alone let them wait on sub-tasks of the chain while ready strips stood behind them
 // (GB300, that order against this one: 8192^2 FP64 181.1 -> 170.0 ms, FP32 96.3 -> 89.4, 4096^2 45.1 -> 42.4, a batch
 // of 64 to 1024 columns FP64 15.4 -> 11.7, FP32 8.5 -> 8.0; scanning ahead of the head instead costs more than it
-// finds, 8192^2 186 ms with 1024 entries).  A sub-task is started after the ones it depends on: the order
-// is topological.  Sub-tasks are numbered topologically on input.
+// finds, 8192^2 186 ms with 1024 entries).  The modelled times are not exact: a quarter of the latest start that delays
+// nothing is added to the start, which lets the sub-tasks with no slack overtake the others (8355 x 473 FP32, FlatTS, tiles
+// of 64: up to 8 % slower without it; times wrong by 20 % cost no more than 1 % with it, in simulations of the traces).
+// Both numbers grow along a dependency: the order is topological.  Sub-tasks are numbered topologically on input.
 static std::vector<int32_t> list_schedule(const std::vector<int64_t>& time, const std::vector<int64_t>& bottom,
                                           const std::vector<int64_t>& dep_begin, const std::vector<int32_t>& deps) {
   constexpr int kWorkers = 152;
@@ -557,6 +596,8 @@ static std::vector<int32_t> list_schedule(const std::vector<int64_t>& time, cons
   std::priority_queue<Item, std::vector<Item>, std::greater<Item>> running;      // (end, number)
   for (int32_t y = 0; y < n; ++y)
     if (open[y] == 0) ready.push({bottom[y], -y});
+  std::vector<int64_t> key(n);
+  const int64_t longest = n > 0 ? *std::max_element(bottom.begin(), bottom.end()) : 0;
   order.reserve(n);
   int64_t now = 0;
   for (int idle = kWorkers;;) {
@@ -564,6 +605,7 @@ static std::vector<int32_t> list_schedule(const std::vector<int64_t>& time, cons
       const int32_t y = -ready.top().second;
       ready.pop();
       order.push_back(y);
+      key[y] = now + (longest - bottom[y]) / 4;
       running.push({now + time[y], y});
     }
     if (running.empty()) break;
@@ -574,6 +616,7 @@ static std::vector<int32_t> list_schedule(const std::vector<int64_t>& time, cons
         if (--open[succ[e]] == 0) ready.push({bottom[succ[e]], -succ[e]});
     }
   }
+  std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return key[a] < key[b]; });
   return order;
 }
 
@@ -670,7 +713,7 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
         wr.push_back(it.t(slot, b));
         const int64_t rows = kind == PK_GE ? nb - (int64_t)b * ib : (kind == PK_TS ? nb : (int64_t)(b + 1) * ib);
         d.op = make_op(PF, lq, false, 0, b, kind);
-        last = g.add(d, sub_time(12 * ib2 * rows, W_PF_GE + kind, rows, ib, 1, esize, prio, digits), rd, wr, -1);
+        last = g.add(d, sub_time(12 * ib2 * rows, W_PF_GE + kind, rows, nb, ib, esize, prio, digits), rd, wr, -1);
         // PU(b, s)
         for (int s = b + 1; s < nblk; ++s) {
           rd.clear();
@@ -691,7 +734,7 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
           }
           rd.push_back(it.t(slot, b));
           d.op = make_op(PU, lq, false, s, b, kind);
-          last = g.add(d, sub_time(6 * ib2 * rows, W_PU_GE + kind, rows, ib, 1, esize, prio, digits), rd, wr, -1);
+          last = g.add(d, sub_time(6 * ib2 * rows, W_PU_GE + kind, rows, nb, ib, esize, prio, digits), rd, wr, -1);
         }
       }
       panel_last[x] = last;
@@ -716,7 +759,7 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
           }
         }
         d.op = make_op(t.type, lq, false, s, 0, 0);
-        g.add(d, sub_time(per_strip, t.type == UNMQR ? W_UNMQR : (t.type == TSMQR ? W_TSMQR : W_TTMQR), nb, ib, nblk,
+        g.add(d, sub_time(per_strip, t.type == UNMQR ? W_UNMQR : (t.type == TSMQR ? W_TSMQR : W_TTMQR), nb, nb, ib,
                           esize, prio, digits),
               rd, wr, panel_last[owner]);
       }
@@ -1099,18 +1142,6 @@ void merge_programs(const std::vector<const Plan*>& plans, std::vector<DevTask>*
 }
 
 namespace {
-
-// Measured mean sub-task times of the executor, per storage precision and (nb, ib): see
-// autotune_table.inc for the command that writes them.  Classes: PF GE / TS / TT, PU GE / TS / TT,
-// UNMQR / TSMQR / TTMQR update strips.
-struct AutotuneRow {
-  int esize, nb, ib;
-  double us[9];
-};
-const AutotuneRow kAutotuneTable[] = {
-#include "autotune_table.inc"
-    {0, 0, 0, {0, 0, 0, 0, 0, 0, 0, 0, 0}},   // end marker
-};
 
 // Fallback model when the table has no row for this precision: padded Table 1 work over the relative
 // efficiency of the tile size in batches (FP64, GB300: FlatTS batches of nb = 32 / 64 / 128 ran at
