@@ -27,6 +27,7 @@
 #ifndef BD_EXEC_PART
 #define BD_EXEC_PART 0
 #endif
+#include <type_traits>
 #include <cstdio>
 
 #include "kernels.cuh"

@@ -40,11 +40,16 @@ __device__ __forceinline__ double recip_series(double x) {
   const double y = (double)__frcp_rn((float)x), e = fma(-x, y, 1.0);
   return fma(y, fma(e, e, e), y);
 }
+__device__ __forceinline__ float rsqrt_approx(float x) {     // (rsqrtf, for normal x)
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 // m^(-1/2) 2^58 for m = x 2^-62 in [2^-7, 1): y0 = Y 2^-20 from the FP32 approximation, then y0 (1 - e)^(-1/2) with
 // e = 1 - m y0^2 (below 2^-18) up to e^2.  Integers: a chain of FP64 operations on one warp takes about 2k cycles here.
 __device__ __forceinline__ int64_t rsqrt_q58(int64_t x) {
   const float f = (float)(uint32_t)(x >> 31) * 0x1p-31f;
-  const uint32_t Y = __float2uint_rn(rsqrtf(f) * 0x1p20f);
+  const uint32_t Y = __float2uint_rn(rsqrt_approx(f) * 0x1p20f);
   const int64_t e = ((int64_t)1 << 56) - (int64_t)__umul64hi((uint64_t)x << 2, ((uint64_t)Y * Y) << 16);
   const int es = (int)(e >> 8);
   const int64_t c = (e >> 1) + ((3 * (((int64_t)es * es) >> 3)) >> 40);
@@ -53,7 +58,7 @@ __device__ __forceinline__ int64_t rsqrt_q58(int64_t x) {
 // u^-1 2^57 for |u| = |x| 2^-61 in [2^-4, 2): the same with y0 = R 2^-19 and e = 1 - |u| y0
 __device__ __forceinline__ int64_t recip_q57(int64_t x) {
   const uint64_t a = x < 0 ? (uint64_t)0 - (uint64_t)x : (uint64_t)x;
-  const uint32_t R = __float2uint_rn(__frcp_rn((float)(uint32_t)(a >> 30) * 0x1p-31f) * 0x1p19f);
+  const uint32_t R = __float2uint_rn(__fdividef(1.0f, (float)(uint32_t)(a >> 30) * 0x1p-31f) * 0x1p19f);
   const int64_t e = ((int64_t)1 << 58) - (int64_t)__umul64hi(a << 2, (uint64_t)R << 40);
   const int es = (int)(e >> 10);
   const int64_t c = e + (((int64_t)es * es) >> 38);
@@ -93,28 +98,27 @@ __device__ __forceinline__ void inverse32(const double* G, const double* d, doub
   }
   __syncthreads();
 #pragma unroll
-  for (int h = 8; h < 32; h *= 2) {    // T12 = -T11 (G12 T22)
-    const int i = tid & (h - 1), j = (tid / h) & (h - 1), c = tid / (h * h) * 2 * h;
+  for (int h = 8; h < 32; h *= 2) {    // T12 = -T11 (G12 T22); the zeros of the triangles T22 and T11 are skipped
+    const int lo = tid & (h - 1), hi = (tid / h) & (h - 1), c = tid / (h * h) * 2 * h, base = tid - (tid & (h * h - 1));
     const bool on = c < 32;
-    double s0 = 0.0, s1 = 0.0;
-    if (on) {
-#pragma unroll
-      for (int t = 0; t < h; t += 2) {
-        s0 = fma(G[c + i + (c + h + t) * 32], T[c + h + t + (c + h + j) * 32], s0);
-        s1 = fma(G[c + i + (c + h + t + 1) * 32], T[c + h + t + 1 + (c + h + j) * 32], s1);
+    if (on) {                          // a warp has the columns hi up to
+      const int last = (((tid | 31) / h) & (h - 1));
+      double s0 = 0.0, s1 = 0.0;
+      for (int t = 0; t <= last; t += 2) {
+        s0 = fma(G[c + lo + (c + h + t) * 32], T[c + h + t + (c + h + hi) * 32], s0);
+        s1 = fma(G[c + lo + (c + h + t + 1) * 32], T[c + h + t + 1 + (c + h + hi) * 32], s1);
       }
-      Y[tid] = s0 + s1;
+      Y[base + lo * h + hi] = s0 + s1;
     }
     __syncthreads();
-    if (on) {
-      const double* y = Y + (tid - (tid & (h * h - 1))) + j * h;
-      s0 = s1 = 0.0;
-#pragma unroll
-      for (int t = 0; t < h; t += 2) {
-        s0 = fma(T[c + i + (c + t) * 32], y[t], s0);
-        s1 = fma(T[c + i + (c + t + 1) * 32], y[t + 1], s1);
+    if (on) {                          // a warp has the rows hi from
+      const int first = (((tid & ~31) / h) & (h - 1)) & ~1;
+      double s0 = 0.0, s1 = 0.0;
+      for (int t = first; t < h; t += 2) {
+        s0 = fma(T[c + hi + (c + t) * 32], Y[base + t * h + lo], s0);
+        s1 = fma(T[c + hi + (c + t + 1) * 32], Y[base + (t + 1) * h + lo], s1);
       }
-      T[c + i + (c + h + j) * 32] = -(s0 + s1);
+      T[c + hi + (c + h + lo) * 32] = -(s0 + s1);
     }
     __syncthreads();
   }
@@ -238,8 +242,8 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
     return true;
   };
   const int arow = 2 * warp;          // thread (warp, lane): rows arow, arow + 1 of column lane of the 32 x 32 matrices
-  auto sum_partials = [&](int k) {
-    const int o = (arow + k) * 33 + lane;
+  auto sum_partials = [&](int row) {
+    const int o = row * 33 + lane;
     return P[o] + P[o + 32 * 33] + P[o + 64 * 33] + P[o + 96 * 33];
   };
 
@@ -249,58 +253,133 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
   gram_partials<true>(P, tq, 24);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   if (!__syncthreads_and(ok ? 1 : 0)) return fail();
-  int64_t m[2] = {sum_partials(0), sum_partials(1)};
-  int64_t bt[2] = {Bs[arow * 33 + lane], Bs[(arow + 1) * 33 + lane]};
-  __syncthreads();
   // ---- Cholesky of M with the elimination of the top block -------------------------------------------
-  // one barrier a step: the warp of row j forms r_j and U_j, then every warp updates its two rows
-#pragma unroll 1
-  for (int j = 0; j < kb; ++j) {
-    if (warp == (j >> 1)) {
-      const int64_t mj = (j & 1) ? m[1] : m[0], bj = (j & 1) ? bt[1] : bt[0];
-      const int64_t mjj = __shfl_sync(kFull, mj, j), al = __shfl_sync(kFull, bj, j);
-      const int64_t rc = __mul64hi(mj << 1, rsqrt_q58(mjj) << 1) << 4;           // 2^62
-      const int64_t u = bj - (al < 0 ? rc >> 1 : -(rc >> 1));                    // 2^61
-      if (lane >= j) {
-        Rw[j * 32 + lane] = split31(rc);
-        Uf[j * 32 + lane] = u;
-      }
-      if (ge) {
-        const int64_t d = recip_q57(__shfl_sync(kFull, u, j));
-        if (lane > j) Ww[j * 32 + lane] = split31(__mul64hi(u << 1, d << 2));   // (|d| < 2^(57 + 3.5))
-        if (lane == 0) dinv[j] = d;
-      }
-      if (lane == 0) {
-        neg[j] = al < 0;
-        if (mjj < (int64_t)1 << 55 || mjj - mul62(al << 1, al << 1) < (int64_t)1 << 42) *refuse = 1;
-      }
-    }
-    __syncthreads();
-    if (arow + 1 > j) {
-      const int2 zero = make_int2(0, 0), rb = lane > j ? Rw[j * 32 + lane] : zero;
-      const int4 ra = *reinterpret_cast<const int4*>(Rw + j * 32 + arow);
-      if (arow > j) m[0] -= mul_hi62(make_int2(ra.x, ra.y), rb);
-      m[1] -= mul_hi62(make_int2(ra.z, ra.w), rb);
-      if (ge) {
-        const int2 wb = lane > j ? Ww[j * 32 + lane] : zero;
+  // Stage s (one barrier each) takes steps j = 2 s and j + 1.  Warp 0 runs the chain: it applies the pair before to rows
+  // j, j + 1 and forms r, U and U / U_jj of both.  The other warps apply that pair to the rows below, two a warp, and
+  // the owner of the next pair hands its rows over, so the chain (its latencies: about 220 cycles for a reciprocal
+  // square root, 190 for a reciprocal) runs beside their work.  Rows 0 .. 7, done with first, are on warp 0's
+  // scheduler.  (Every warp forming its own rows of r and U after a barrier a step: 56.7k cycles for a GE block and 28k for TS,
+  // against 37k and 23k.)
+  const int pr = (warp & 3) == 0 ? warp >> 2 : 3 + 3 * (warp >> 2) + (warp & 3), erow = 2 * pr;
+  int64_t m[2], bt[2];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          const int64_t bij = __shfl_sync(kFull, bt[k], j);
-          if (arow + k > j) {
-            if (lane == 0) Bs[(arow + k) * 33 + j] = bij;    // l_ij U_jj
-            bt[k] -= mul_hi57(split31(bij), wb);
-          }
-        }
-      }
-    }
+  for (int k = 0; k < 2; ++k) {
+    m[k] = sum_partials(erow + k);
+    bt[k] = Bs[(erow + k) * 33 + lane];
   }
   __syncthreads();
+  int64_t* H = reinterpret_cast<int64_t*>(sm + kPanG);       // rows handed over: two buffers of m, m, bt, bt
+  auto eliminate = [&](auto is_ge) {
+    constexpr bool kGe = decltype(is_ge)::value;
+    const int2 zero = make_int2(0, 0);
+    if (warp == 0) {
+      int2 rs[2] = {zero, zero}, ws[2] = {zero, zero};
+#pragma unroll 1
+      for (int j = 0; j < kb; j += 2) {
+        if (j > 0) {
+          const int64_t* h = H + (j & 2) * 64 + lane;
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            m[k] = h[32 * k];
+            bt[k] = h[64 + 32 * k];
+          }
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+              m[k] -= mul_hi62(make_int2(__shfl_sync(kFull, rs[q].x, j + k), __shfl_sync(kFull, rs[q].y, j + k)), rs[q]);
+            if (kGe) {
+#pragma unroll
+              for (int k = 0; k < 2; ++k) {
+                const int64_t bij = __shfl_sync(kFull, bt[k], j - 2 + q);
+                if (lane == 0) Bs[(j + k) * 33 + j - 2 + q] = bij;       // l_ij U_jj
+                bt[k] -= mul_hi57(split31(bij), ws[q]);
+              }
+            }
+          }
+        }
+        const int64_t m0 = __shfl_sync(kFull, m[0], j), al0 = __shfl_sync(kFull, bt[0], j);
+        const int64_t rc0 = __mul64hi(m[0] << 1, rsqrt_q58(m0) << 1) << 4;               // 2^62
+        rs[0] = lane > j ? split31(rc0) : zero;
+        m[1] -= mul_hi62(make_int2(__shfl_sync(kFull, rs[0].x, j + 1), __shfl_sync(kFull, rs[0].y, j + 1)), rs[0]);
+        const int64_t m1 = __shfl_sync(kFull, m[1], j + 1), y1 = rsqrt_q58(m1);
+        const int64_t u0 = bt[0] - (al0 < 0 ? rc0 >> 1 : -(rc0 >> 1));                   // 2^61
+        int64_t d0 = 0, b10 = 0;
+        if (kGe) {
+          d0 = recip_q57(__shfl_sync(kFull, u0, j));                                     // |d| < 2^(57 + 3.5)
+          ws[0] = lane > j ? split31(__mul64hi(u0 << 1, d0 << 2)) : zero;
+          b10 = __shfl_sync(kFull, bt[1], j);
+          bt[1] -= mul_hi57(split31(b10), ws[0]);
+        }
+        const int64_t rc1 = __mul64hi(m[1] << 1, y1 << 1) << 4;
+        const int64_t al1 = __shfl_sync(kFull, bt[1], j + 1);
+        const int64_t u1 = bt[1] - (al1 < 0 ? rc1 >> 1 : -(rc1 >> 1));
+        rs[1] = lane > j + 1 ? split31(rc1) : zero;
+        int64_t d1 = 0;
+        if (kGe) {
+          d1 = recip_q57(__shfl_sync(kFull, u1, j + 1));
+          ws[1] = lane > j + 1 ? split31(__mul64hi(u1 << 1, d1 << 2)) : zero;
+          Ww[j * 32 + lane] = ws[0];
+          Ww[j * 32 + 32 + lane] = ws[1];
+        }
+        Rw[j * 32 + lane] = lane == j ? split31(rc0) : rs[0];
+        Rw[j * 32 + 32 + lane] = lane == j + 1 ? split31(rc1) : rs[1];
+        Uf[j * 32 + lane] = u0;
+        Uf[j * 32 + 32 + lane] = u1;
+        if (lane == 0) {
+          if (kGe) {
+            Bs[(j + 1) * 33 + j] = b10;
+            dinv[j] = d0;
+            dinv[j + 1] = d1;
+          }
+          neg[j] = al0 < 0;
+          neg[j + 1] = al1 < 0;
+          if (min(m0, m1) < (int64_t)1 << 55 || min(m0 - mul62(al0 << 1, al0 << 1), m1 - mul62(al1 << 1, al1 << 1)) < (int64_t)1 << 42)
+            *refuse = 1;
+        }
+        __syncthreads();
+      }
+    } else {
+#pragma unroll 1
+      for (int j = 0; j < kb; j += 2) {
+        if (erow > j && j > 0) {             // steps j - 2 and j - 1
+#pragma unroll
+          for (int q = j - 2; q < j; ++q) {
+            const int2 rb = Rw[q * 32 + lane];
+            const int4 ra = *reinterpret_cast<const int4*>(Rw + q * 32 + erow);
+            m[0] -= mul_hi62(make_int2(ra.x, ra.y), rb);
+            m[1] -= mul_hi62(make_int2(ra.z, ra.w), rb);
+            if (kGe) {
+              const int2 wb = Ww[q * 32 + lane];
+#pragma unroll
+              for (int k = 0; k < 2; ++k) {
+                const int64_t bij = __shfl_sync(kFull, bt[k], q);
+                if (lane == 0) Bs[(erow + k) * 33 + q] = bij;
+                bt[k] -= mul_hi57(split31(bij), wb);
+              }
+            }
+          }
+        }
+        if (erow == j + 2) {
+          int64_t* h = H + (erow & 2) * 64 + lane;
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            h[32 * k] = m[k];
+            h[64 + 32 * k] = bt[k];
+          }
+        }
+        __syncthreads();
+      }
+    }
+  };
+  if (ge) eliminate(std::true_type{});
+  else eliminate(std::false_type{});
   if (*refuse) return false;           // (uniform: not written again)
   // ---- U^{-1}, its digits ------------------------------------------------------------------------
 #pragma unroll
   for (int k = 0; k < 2; ++k)
-    G[arow + k + lane * 32] = (lane > arow + k && lane < kb) ? (double)Uf[(arow + k) * 32 + lane] * 0x1p-61 : 0.0;
-  if (tid < 32) diag[tid] = tid < kb ? recip_series((double)Uf[tid * 33] * 0x1p-61) : 0.0;
+    G[arow + k + lane * 32] = (lane > arow + k && lane < kb) ? from_fixed(Uf[(arow + k) * 32 + lane], 61) : 0.0;
+  if (tid < 32) diag[tid] = tid < kb ? recip_series(from_fixed(Uf[tid * 33], 61)) : 0.0;
   __syncthreads();
   inverse32(G, diag, Td, G + 1024);
   {
@@ -402,11 +481,11 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
   if (!__syncthreads_and(ok ? 1 : 0)) return fail();
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
-    const double v = (double)sum_partials(k) * 0x1p-61;
+    const double v = from_fixed(sum_partials(arow + k), 61);
     G[arow + k + lane * 32] = v;
-    if (arow + k == lane) diag[lane] = lane < kb ? 2.0 * recip_series(ge ? v : 1.0 + v) : 0.0;
   }
   __syncthreads();
+  if (tid < 32) diag[tid] = tid < kb ? 2.0 * recip_series(ge ? G[tid * 33] : 1.0 + G[tid * 33]) : 0.0;
   inverse32(G, diag, Td, G + 1024);
   for (int o = tid; o < kb * kb; o += kThreads)
     stg(Tg + (size_t)c0 * ib + o, Td[kb == 32 ? o : o % kb + o / kb * 32]);
