@@ -550,18 +550,43 @@ __device__ void factor_panel(int mode, E* P, int lp, int rows, int kb, E* Rt, in
         __syncwarp();
         if (lane == 0 && !pairs) scalars(c, part);
       }
-    } else if (refl && sizeof(E) == 8) {   // FP64: one column per pass (the FP64 pipe is the limit)
+    } else if (refl && sizeof(E) == 8) {
+      // FP64: a scheduler issues an FP64 instruction of a warp every 64 cycles, so the work is counted in them.  Up to four
+      // columns a pass: their sums are reduced together (lane bits 16 and 8 choose the column, six additions instead of
+      // twenty, each sum in the order of warp_sum) and their scalars formed once.  Warps 4, 8, 12 stay idle: they share
+      // warp 0's scheduler, whose chain every column waits for.  (3001 x 1537 18.4 -> 17.8 ms, a
+      // batch of 64 11.3 -> 10.7: the last blocks of their GE panels.)
       const E taue = tauE;
-      for (int c = jj + 2 + (warp - 1); c < kb; c += kWarps - 1) {
-        E sum = E(0);
-        for (int r = t0 + lane; r < t1; r += 32) sum += P[r + jj * lp] * P[r + c * lp];
-        sum = warp_sum(sum);
-        E* top = (mode == PM_GE) ? &P[jj + c * lp] : &Rt[jj + c * lrt];
-        const E wv = *top + se * sum;
-        __syncwarp();
-        if (lane == 0) *top = *top - taue * wv;
-        const E tw = taue * wv * se;
-        for (int r = t0 + lane; r < t1; r += 32) P[r + c * lp] -= P[r + jj * lp] * tw;
+      const int worker = warp - 1 - (warp >> 2), left = kb - (jj + 2), group = min(4, (left + 2) / 3);
+      if (warp & 3) {
+        const bool b16 = lane & 16, b8 = lane & 8;
+        for (int cg = jj + 2 + group * worker; cg < kb; cg += group * (kWarps * 3 / 4)) {
+          const int nc = min(group, kb - cg);
+          E s[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            s[k] = E(0);
+            if (k < nc)
+              for (int r = t0 + lane; r < t1; r += 32) s[k] += P[r + jj * lp] * P[r + (cg + k) * lp];
+          }
+          const E u0 = (b16 ? s[1] : s[0]) + __shfl_xor_sync(kFull, b16 ? s[0] : s[1], 16);
+          const E u1 = (b16 ? s[3] : s[2]) + __shfl_xor_sync(kFull, b16 ? s[2] : s[3], 16);
+          E sum = (b8 ? u1 : u0) + __shfl_xor_sync(kFull, b8 ? u0 : u1, 8);
+#pragma unroll
+          for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+          const int k = (b16 ? 1 : 0) + (b8 ? 2 : 0), c = cg + min(k, nc - 1);
+          E* top = (mode == PM_GE) ? &P[jj + c * lp] : &Rt[jj + c * lrt];
+          const E wv = *top + se * sum;
+          __syncwarp();
+          if ((lane & 7) == 0 && k < nc) *top = *top - taue * wv;
+          const E tw = taue * wv * se;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const E twq = __shfl_sync(kFull, tw, (q & 1) * 16 + (q >> 1) * 8);
+            if (q < nc)
+              for (int r = t0 + lane; r < t1; r += 32) P[r + (cg + q) * lp] -= P[r + jj * lp] * twq;
+          }
+        }
       }
     } else if (refl) {
       // FP32: two columns c and c + 7 per pass (independent, so their reductions overlap; a lone last
@@ -622,6 +647,56 @@ __device__ void factor_panel(int mode, E* P, int lp, int rows, int kb, E* Rt, in
   __syncthreads();
 }
 
+#if BD_EXEC_PART == 1
+// T = the inverse of the 32 x 32 upper triangular matrix with G above its diagonal (column-major, only that part is read)
+// and reciprocal diagonal d; Y: 512 doubles of scratch.  As t_from_gram, for 512 threads with fixed bounds: 20k cycles
+// there, most of it latency and index arithmetic.
+__device__ __forceinline__ void inverse32(const double* G, const double* d, double* T, double* Y) {
+  const int tid = threadIdx.x;
+  for (int o = tid; o < 1024; o += kThreads) T[o] = 0.0;
+  __syncthreads();
+  if (tid < 32) {                      // the diagonal 8 x 8 blocks, a row a thread
+    const int o = tid & 24, a = tid & 7;
+    double t[8], acc[8];
+#pragma unroll
+    for (int l = 0; l < 8; ++l) acc[l] = 0.0;
+#pragma unroll
+    for (int l = 0; l < 8; ++l) {
+      t[l] = l < a ? 0.0 : (l == a ? d[o + l] : -d[o + l] * acc[l]);
+#pragma unroll
+      for (int k = l + 1; k < 8; ++k) acc[k] = fma(t[l], G[o + l + (o + k) * 32], acc[k]);
+      T[o + a + (o + l) * 32] = t[l];
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 8; h < 32; h *= 2) {    // T12 = -T11 (G12 T22); the zeros of the triangles T22 and T11 are skipped
+    const int lo = tid & (h - 1), hi = (tid / h) & (h - 1), c = tid / (h * h) * 2 * h, base = tid - (tid & (h * h - 1));
+    const bool on = c < 32;
+    if (on) {                          // a warp has the columns hi up to
+      const int last = (((tid | 31) / h) & (h - 1));
+      double s0 = 0.0, s1 = 0.0;
+      for (int t = 0; t <= last; t += 2) {
+        s0 = fma(G[c + lo + (c + h + t) * 32], T[c + h + t + (c + h + hi) * 32], s0);
+        s1 = fma(G[c + lo + (c + h + t + 1) * 32], T[c + h + t + 1 + (c + h + hi) * 32], s1);
+      }
+      Y[base + lo * h + hi] = s0 + s1;
+    }
+    __syncthreads();
+    if (on) {                          // a warp has the rows hi from
+      const int first = (((tid & ~31) / h) & (h - 1)) & ~1;
+      double s0 = 0.0, s1 = 0.0;
+      for (int t = first; t < h; t += 2) {
+        s0 = fma(T[c + hi + (c + t) * 32], Y[base + t * h + lo], s0);
+        s1 = fma(T[c + hi + (c + t + 1) * 32], Y[base + (t + 1) * h + lo], s1);
+      }
+      T[c + hi + (c + h + lo) * 32] = -(s0 + s1);
+    }
+    __syncthreads();
+  }
+}
+#endif
+
 // T from the reflectors' tau and the strict upper part of G = V^T V (kb x kb, ld kb; kb x kb more are scratch): the
 // inverse of the upper triangular matrix with diagonal 1 / tau and G above it.  The forward recurrence
 // T[l,l] = tau_l, T[0:l, l] = -tau_l T[0:l, 0:l] G[0:l, l] inside diagonal blocks of 8 columns (all blocks at once),
@@ -630,6 +705,12 @@ __device__ void factor_panel(int mode, E* P, int lp, int rows, int kb, E* Rt, in
 template <typename E>
 __device__ void t_from_gram(int kb, const double* tau_s, E* Tb, int ldt, E* G) {
   E* Y = G + kb * kb;
+#if BD_EXEC_PART == 1
+  if (kb == 32 && ldt == 32) {
+    inverse32(G, tau_s, Tb, Y);
+    return;
+  }
+#endif
   constexpr int kB0 = 8;
   for (int o = threadIdx.x; o < kb * kb; o += kThreads) Tb[(o % kb) + (o / kb) * ldt] = E(0);
   __syncthreads();

@@ -76,54 +76,6 @@ __device__ __forceinline__ int64_t mul_hi57(int2 a, int2 b) {       // a b 2^-57
   return (int64_t)((uint64_t)((int64_t)a.x * b.x) << 5) + (mid >> 26);
 }
 
-// T = the inverse of the 32 x 32 upper triangular matrix with G above its diagonal (column-major, only that part is read)
-// and reciprocal diagonal d; Y: 512 doubles of scratch.  As t_from_gram, for 512 threads with fixed bounds: 20k cycles
-// there, most of it latency and index arithmetic.
-__device__ __forceinline__ void inverse32(const double* G, const double* d, double* T, double* Y) {
-  const int tid = threadIdx.x;
-  for (int o = tid; o < 1024; o += kThreads) T[o] = 0.0;
-  __syncthreads();
-  if (tid < 32) {                      // the diagonal 8 x 8 blocks, a row a thread
-    const int o = tid & 24, a = tid & 7;
-    double t[8], acc[8];
-#pragma unroll
-    for (int l = 0; l < 8; ++l) acc[l] = 0.0;
-#pragma unroll
-    for (int l = 0; l < 8; ++l) {
-      t[l] = l < a ? 0.0 : (l == a ? d[o + l] : -d[o + l] * acc[l]);
-#pragma unroll
-      for (int k = l + 1; k < 8; ++k) acc[k] = fma(t[l], G[o + l + (o + k) * 32], acc[k]);
-      T[o + a + (o + l) * 32] = t[l];
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int h = 8; h < 32; h *= 2) {    // T12 = -T11 (G12 T22); the zeros of the triangles T22 and T11 are skipped
-    const int lo = tid & (h - 1), hi = (tid / h) & (h - 1), c = tid / (h * h) * 2 * h, base = tid - (tid & (h * h - 1));
-    const bool on = c < 32;
-    if (on) {                          // a warp has the columns hi up to
-      const int last = (((tid | 31) / h) & (h - 1));
-      double s0 = 0.0, s1 = 0.0;
-      for (int t = 0; t <= last; t += 2) {
-        s0 = fma(G[c + lo + (c + h + t) * 32], T[c + h + t + (c + h + hi) * 32], s0);
-        s1 = fma(G[c + lo + (c + h + t + 1) * 32], T[c + h + t + 1 + (c + h + hi) * 32], s1);
-      }
-      Y[base + lo * h + hi] = s0 + s1;
-    }
-    __syncthreads();
-    if (on) {                          // a warp has the rows hi from
-      const int first = (((tid & ~31) / h) & (h - 1)) & ~1;
-      double s0 = 0.0, s1 = 0.0;
-      for (int t = first; t < h; t += 2) {
-        s0 = fma(T[c + hi + (c + t) * 32], Y[base + t * h + lo], s0);
-        s1 = fma(T[c + hi + (c + t + 1) * 32], Y[base + (t + 1) * h + lo], s1);
-      }
-      T[c + hi + (c + h + lo) * 32] = -(s0 + s1);
-    }
-    __syncthreads();
-  }
-}
-
 // Factors inner block b of a panel task as task_panel_factor does, and publishes it in vd if that is given; false:
 // refused, nothing written.
 __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, double* X, double* A, int tr, double* Tg, int nb,
