@@ -52,19 +52,20 @@ WORKLOADS = {
                                "+ adjoint (dL/dA from a N(0,1) band gradient W, L = <W, B>)"),
 }
 # FP64 peak of the GB300 from its unit counts and clock: 152 SMs x 2 FP64 FMA/clock/SM (4 flops) x
-# 2070 MHz = 1258.6 GFLOP/s.  Reported beside the measured peaks; the roofline divides by the measured
-# DFMA-loop rate (bidiag_measure_fp64_peaks), the FP64 unit the reduction's contractions run on.
+# 2070 MHz = 1258.6 GFLOP/s.  Reported beside the measured peaks; the roofline of the adjoint divides by the
+# measured DFMA-loop rate (bidiag_measure_fp64_peaks), the FP64 unit its contractions run on.
 FP64_DERIVED_GFLOPS = 152 * 4 * 2.070
-# DRAM bytes (read + write) of one executor launch on the 8192^2 Auto workload, from the ncu capture
-# summarised under profiles/exec_kernel_square8192_launches.md (set to None when the kernel changes).
-EXEC_TRAFFIC_BYTES = 11638296576 + 11605000704
+# An FP64 reduction's contractions run as exact products of 8-bit digits on the f16 tensor pipe: seven digits an
+# operand, of whose pairs the 34 with i + j < 8 count (the rest weighs less than the rounding).
+DIGIT_PRODUCTS = 34
 CPU_SAMPLE_SECONDS = 12.0
 
 
 def measure_peaks(G, torch, local, f32):
     """Measured denominators, taken on this GPU before the timed region: the FP64 DFMA and FP64 MMA
-    loops of the library's probe, cuBLAS DGEMM (torch.matmul, FP64, 4096^3) and, for the split-precision
-    form, cuBLAS TF32 (torch.matmul, FP32 with TF32 allowed, 8192^3); best of several runs each."""
+    loops of the library's probe, cuBLAS DGEMM (torch.matmul, FP64, 4096^3) and cuBLAS BF16 (8192^3) or, for
+    the split-precision form, cuBLAS TF32 (torch.matmul, FP32 with TF32 allowed, 8192^3); best of several
+    runs each."""
     out = {}
     fma, mma = G.bidiag_measure_fp64_peaks(local, None)
     out["fp64_dfma_loop_gflops"] = fma
@@ -88,6 +89,8 @@ def measure_peaks(G, torch, local, f32):
         return best
 
     out["fp64_dgemm_gflops"] = best_rate(torch.float64, 4096, 3)
+    if not f32:
+        out["bf16_gemm_gflops"] = best_rate(torch.bfloat16, 8192, 10)
     if f32:
         prev = torch.backends.cuda.matmul.allow_tf32
         torch.backends.cuda.matmul.allow_tf32 = True
@@ -99,13 +102,17 @@ def measure_peaks(G, torch, local, f32):
     return out
 
 
-def roofline_peak(peaks, f32):
-    """(peak GFLOP/s, bound, source) of the reduction's executor: FP64 storage against the measured
-    DFMA loop; FP32 storage against the measured TF32 GEMM rate over the three TF32 products that
+def roofline_peak(peaks, f32, adjoint=False):
+    """(peak GFLOP/s, bound, source) of the executor: FP64 reductions against the measured BF16 GEMM rate
+    (that of the f16 pipe) over the digit products that make one useful product, their adjoint against the
+    measured DFMA loop; FP32 storage against the measured TF32 GEMM rate over the three TF32 products that
     make one useful product."""
     if f32:
         return (peaks["tf32_gemm_gflops"] / 3.0, "tensor",
                 "measured: cuBLAS TF32 GEMM 8192^3 (torch.matmul) / 3 products per useful flop")
+    if not adjoint:
+        return (peaks["bf16_gemm_gflops"] / DIGIT_PRODUCTS, "tensor",
+                "measured: cuBLAS BF16 GEMM 8192^3 (torch.matmul) / 34 digit products per useful product")
     return (peaks["fp64_dfma_loop_gflops"], "alu",
             "measured: FP64 DFMA loop (bidiag_measure_fp64_peaks), all SMs")
 
@@ -601,7 +608,7 @@ def run_grad(args, w, base, config, world, rank, local, device, G, torch):
     alg = table1_flops(G, m, n, nb, G.TREES[tree], G.VARIANTS[w["variant"]], 1)
     bwd_flops = 3.0 * alg
     achieved = bwd_flops / (bwd_ms * 1e-3) / 1e9
-    peak, bound, src = roofline_peak(peaks, f32)
+    peak, bound, src = roofline_peak(peaks, f32, adjoint=True)
     line = dict(base, config=config, dtype="f32" if f32 else "f64", value=value, ms_per_step=ms_per_step,
                 e2e={"value": world * flops / e2e_s / 1e12 if e2e_s else None, "unit": "TFLOP/s",
                      "h2d_bytes_per_step": m * n * A.element_size(), "d2h_bytes_per_step": m * n * A.element_size()},
@@ -1038,7 +1045,7 @@ def main():
                      "h2d_bytes_per_step": m * n * A.element_size(),
                      "d2h_bytes_per_step": (nb + 1) * n * A.element_size()},
                 roofline={"bound": bound, "achieved": achieved, "peak": peak, "unit": unit,
-                          "frac": achieved / peak, "traffic": EXEC_TRAFFIC_BYTES if (not f32 and w["name"] == "square8192" and args.tree == "auto") else None,
+                          "frac": achieved / peak, "traffic": None,
                           "kernel": "exec_kernel (persistent dataflow executor)", "algorithmic_flops": alg,
                           "peak_source": peak_src, "peaks_measured": peaks},
                 exec_ms=exec_ms, gpu_launches=3 * args.steps, clocks=clocks)

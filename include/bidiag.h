@@ -86,11 +86,10 @@ enum {
                                      and scanning costs more than it finds (8192^2 170 against 186 ms).
                                      Results do not depend on it: the program orders every
                                      access to shared data, the window only changes timing */
-  BIDIAG_OPT_PRIORITY = 10        /* queue order of the device program, by bottom level (longest weighted
-                                     path to the end) with sub-task weights 1 = Table 1 flops times the
-                                     measured time per flop of each sub-task kind (default), 0 = flops
-                                     alone (FP32-storage panel factors twice).  Results do not depend on
-                                     it */
+  BIDIAG_OPT_PRIORITY = 10        /* queue order of the device program: that of a list schedule by longest
+                                     path to the end, with sub-task times 1 = modelled from measurements
+                                     (default), 0 = Table 1 flops (FP32-storage panel factors twice).
+                                     Results do not depend on it */
 };
 
 /* Task type codes of the canonical task list (GELQT etc. are the same codes in LQ phases). */

@@ -9,7 +9,9 @@
 // an orientation flag `tr`, so GELQT/UNMLQ/... are GEQRT/UNMQR/... on the transposed geometry.
 //
 // FP64: GB300's FP64 units deliver 2 FMA/clock/SM (about 1.2 TFLOP/s per GPU, measured) and FP64 MMA
-// is not faster than DFMA on this part, so the contractions are register-blocked DFMA loops.
+// is not faster than DFMA on this part.  Updates and panel factors of reductions run as exact digit products on
+// the f16 tensor pipe where the sizes fit (update_digits.cuh, panel_digits.cuh); smaller tiles, refused blocks and
+// the adjoint take register-blocked DFMA loops.
 // FP32 storage: the contractions of the updates run on the tensor cores as three TF32 products,
 // a_hi b_hi + a_hi b_lo + a_lo b_hi with a = a_hi + a_lo (a_hi = TF32 round-to-nearest of a, a_lo =
 // TF32 of the remainder), accumulated in FP32 (Markidis et al. 2018; Ootomo and Yokota 2022); the

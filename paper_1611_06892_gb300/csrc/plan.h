@@ -90,7 +90,7 @@ struct Plan {
   int npanels = 0;
   int64_t critical_path = 0;       // Table 1 units
   // device program
-  std::vector<DevTask> dev;        // in queue (priority) order
+  std::vector<DevTask> dev;        // in queue order (a list schedule's)
   std::vector<int32_t> deps;       // indices into dev (queue positions)
   std::vector<int64_t> prio;       // bottom level of each queued sub-task (modelled times)
   std::vector<int64_t> time;       // modelled time of each
