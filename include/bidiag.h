@@ -140,6 +140,11 @@ int bidiag_set_option(bidiag_handle h, int option, int64_t value);
  * in 0..2 (-9), out != NULL (-10).  m < n returns BIDIAG_ERR_UNSUPPORTED (Sec. 3.6: the transposed
  * problem).  *out receives a new result object (free with bidiag_result_free) that owns the band, the
  * reflector store and the canonical task list.  The call enqueues the work and returns.
+ * Where nb ib >= 1024, ib <= 32, nb and ib are multiples of 8 and the strips are not wider than 32 columns, the
+ * factors and updates run on the tensor cores as exact products of 8-bit digits, each column held to 2^-56 of its
+ * norm.  Blocks with rows that are much smaller than the others (below about 2^-8 of the column's scale), with columns
+ * outside [2^-958, 2^977] or with entries that are not finite run in FP64 arithmetic, so that rows keep their own scale
+ * as there.  Squared norms of whole columns have to be in the range of FP64 either way (no scaling, as in the paper).
  */
 int bidiag_band(bidiag_handle h, int64_t m, int64_t n, const double* d_A, int64_t lda,
                 int nb, int ib, int tree, int variant, bidiag_result_t* out);

@@ -17,10 +17,12 @@
 //
 // The Gram matrix squares the condition number: an error of 2^-57 in M (the rounding of the 56-bit digits) becomes
 // 2^-58 / r_jj in R'.  Blocks in which a column's norm falls below 2^-3.5 of its start under the reflectors before it, in
-// which a tail is (nearly) zero (sigma^2 < 2^-20; an exact zero must give H = I), or whose U^{-1} exceeds 2^5, are refused
-// before anything is written and factored column by column (task_panel_factor); so are the square blocks at a GE panel's
-// end, whose last columns are short.  (Backward error against a 113-bit product, 256 rows N(0, 1): 4.6e-16, column by
-// column 8.5e-16; ||Q^T Q - I|| 3e-16 against 8e-16.)
+// which a tail is (nearly) zero (sigma^2 < 2^-20; an exact zero must give H = I), whose U^{-1} exceeds 2^5, or in which X
+// has no entry of 2^-8 or a row with no entry above 2^-6 of its largest (2^-10 for a triangle: its rows have their large
+// entries on the diagonal, in another block; smaller rows would not be held to their own scale, as in
+// update_digits.cuh), are refused before anything is written and factored column by column
+// (task_panel_factor); so are the square blocks at a GE panel's end, whose last columns are short.  (Backward error against
+// a 113-bit product, 256 rows N(0, 1): 4.6e-16, column by column 8.5e-16; ||Q^T Q - I|| 3e-16 against 8e-16.)
 
 #if BD_EXEC_PART == 1
 constexpr int kPanR = kDigC;                        // byte offsets: R's digits (32 rows, 2048 bytes a digit),
@@ -106,6 +108,8 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
   const bool is_top = ti >= 0 && ti < kb;
 
   // ---- load, E_c --------------------------------------------------------------------------------
+  uint32_t* rows = reinterpret_cast<uint32_t*>(sm + kPanG);
+  uint32_t big = 0;                    // largest |X| of the thread's half row
   int64_t cf[16];
   {
     auto load_row = [&](const double* src, int row, bool on, int64_t* v) {
@@ -133,16 +137,26 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
 #pragma unroll
     for (int c = 0; c < 16; ++c) cq[c] = r > cb + c ? 0 : cq[c];          // R's upper triangle (r < kb)
     int E;
-    if (!column_exponents(cf, cq, colE, red, &E, cb + (lane & 15) >= kb)) return false;
+    bool zero;
+    if (!column_exponents(cf, cq, colE, red, &E, &zero, cb + (lane & 15) >= kb)) return false;
     for (int o = tid; o < 32 * 33; o += kThreads) Bs[o] = 0;
     __syncthreads();
     if (tid == 0) *refuse = 0;
+    bool nz = false;
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
       const int sh = 63 - __shfl_sync(kFull, E, c);
+      nz = nz || cf[c] << 1 != 0;
       cf[c] = to_fixed(__longlong_as_double(cf[c]), sh);
       cq[c] = to_fixed(__longlong_as_double(cq[c]), sh);
+      big = max(big, abs_hi(cf[c]));
       if (is_top) Bs[ti * 33 + cb + c] = (ge ? cf[c] : cq[c]) >> 2;       // 2^61
+    }
+    const uint32_t wmax = __reduce_max_sync(kFull, big);
+    const unsigned any = __ballot_sync(kFull, nz);
+    if (lane == 0) {
+      rows[warp] = wmax;
+      rows[16 + warp] = any;
     }
 #pragma unroll
     for (int g = 0; g < 2; ++g) put_digits(sm + kDigV, r, 2 * ch + g, cf + 8 * g);
@@ -201,6 +215,15 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
 
   // ---- M = R^T R + X^T X (2^62) -------------------------------------------------------------------
   fence_sync();
+  {                                    // rows of another scale (every warp finds the same)
+    const uint32_t xmax = __reduce_max_sync(kFull, rows[lane & 15]);
+    const unsigned strong = __ballot_sync(kFull, big >= xmax >> (tt ? 10 : 6));
+    if (lane == 0) rows[32 + warp] = strong;
+    __syncthreads();
+    const int w = lane & 7;
+    const uint32_t weak = (rows[16 + w] | rows[24 + w]) & ~(rows[32 + w] | rows[40 + w]);
+    if (xmax < kSmallRow || __any_sync(kFull, weak != 0)) return false;
+  }
   gram(!ge);
   gram_partials<true>(P, tq, 24);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -405,6 +428,7 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
       cf[c] = cb + c < ti ? min(max((int64_t)__mul64hi(Bs[ti * 33 + cb + c] << 2, dinv[cb + c] << 2) << 4, -one), one)
                           : (cb + c == ti ? one + 1 : 0);
   }
+  bool nz = false;                     // V has an entry in the thread's half row
   if (own && ok) {
 #pragma unroll
     for (int c = 0; c < 16; c += 2) {
@@ -412,6 +436,7 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
       const bool on = cb + c < kb, w0 = on && (ge ? d > 0 : (!tt || d <= 0)), w1 = on && (ge ? d > 1 : (!tt || d <= 1));
       double* p = X + toff(r, c0 + cb + c, nb, tr);
       const double x = from_fixed(cf[c], 62), y = from_fixed(cf[c + 1], 62);
+      nz = nz || x != 0.0 || y != 0.0;
       cf[c] = to_fixed(x, 62);                            // V as it is stored
       cf[c + 1] = to_fixed(y, 62);
       if (tr && w0 && w1) {
@@ -443,7 +468,7 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
     stg(Tg + (size_t)c0 * ib + o, Td[kb == 32 ? o : o % kb + o / kb * 32]);
   if (vd) {
     const double t[2] = {Td[arow + lane * 32], Td[arow + 1 + lane * 32]};
-    publish_t(vd, nb, t, true, reinterpret_cast<uint32_t*>(colS + 96));
+    publish_t(vd, nb, t, true, nz, reinterpret_cast<uint32_t*>(colS));
     wait_image();
   }
   __syncthreads();

@@ -72,9 +72,9 @@ BD_HD inline bool digits_fit(int nb, int ib, int ncols) {
 }
 
 // A published panel block (update_digits.cuh): kDigitCount digits of V, 64 bytes a row, T and a header.
-constexpr int kDigitCount = 7, kDigitTBytes = 32 * 34 * 8;
+constexpr int kDigitCount = 7, kDigitTBytes = 32 * 34 * 8, kDigitHeadBytes = 128;
 BD_HD inline int digit_image_rows(int nb) { return (nb + 15) & ~15; }
-BD_HD inline int64_t digit_block_bytes(int nb) { return (int64_t)kDigitCount * digit_image_rows(nb) * 64 + kDigitTBytes + 128; }
+BD_HD inline int64_t digit_block_bytes(int nb) { return (int64_t)kDigitCount * digit_image_rows(nb) * 64 + kDigitTBytes + kDigitHeadBytes; }
 
 inline int32_t tile_ref(int buf, int64_t idx) { return (int32_t)(((uint32_t)buf << 28) | (uint32_t)idx); }
 

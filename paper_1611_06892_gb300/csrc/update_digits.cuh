@@ -23,6 +23,15 @@
 // Columns that are not finite, or outside [2^-958, 2^977], and blocks whose V or T are out of range are
 // refused; the caller runs them on the FP64 units (task_update).
 //
+// Rows.  FP64 arithmetic keeps a row that is far smaller than the others to its own scale (weighted least squares;
+// rows from 1 to 1e-16: R's rows to 1e-13), fixed point by columns does not.  A block is therefore refused too, before
+// any of it is applied, if it changes a row r that is small and stays small: |C(r, c)| < 2^-8 2^E_c and
+// |V(r, j)| |W2(j, c)| < 2^-10 2^E_c for all j and c; or a pivot row j as small, under a reflector with next to no tail
+// (tau_j > 2 - 2^-14).  Rows of N(0, 1) columns have entries near 2^-4 2^E_c, so that full strips of ordinary matrices
+// never come to the second test (rows_lost).  In strips of fewer than 8 columns a row can be small by chance: there the
+// row of V has to be small too, |V(r, j)| < 2^-8 of the reflector's norm for all j.  Rows that no reflector touches are
+// not written back.
+//
 // Layout.  512 threads: thread t owns columns 16 (t / 256) .. + 15 of row t % 256 of the strip (int64 in registers;
 // with 256 threads of 32 columns the code was bound by its own latencies, two warps a scheduler): TMEM lane = row,
 // so the product V W2 arrives where it is subtracted, and the new digits of the row go to shared memory in 16-byte
@@ -45,8 +54,9 @@ constexpr int kDigT = kDigP + 4 * kDigPStride;      //   and op(T), 32 rows of 3
 constexpr int kDigHead = 2 * kDigN * kDigSlice;     // column exponents, reduction scratch
 constexpr int kDigBytes = kDigHead + 128 + 1024;
 static_assert(kDigW2 + 8 * 2048 <= kDigP + 4 * kDigPStride, "W2 digits fit beside W");
-static_assert(kDigT + 32 * 34 * 8 <= kDigHead, "T fits");
+static_assert(kDigT + 32 * 34 * 8 + kDigitHeadBytes <= kDigHead, "T and the header fit");
 static_assert((kDigW2 & 127) == 0, "operand alignment");
+constexpr int kDigRow = kDigP + 3 * kDigPStride;    // scratch of the tests of rows, between two uses of that slot
 constexpr int kDigTmem = 512;
 constexpr int kDigTBytes = 32 * 34 * 8;
 static_assert(kDigTBytes == kDigitTBytes && kDigN == kDigitCount, "published blocks");
@@ -150,11 +160,11 @@ __device__ __forceinline__ float transpose_sum16(float* v) {
 }
 
 // E_c of the columns whose entries the CTA's threads hold as FP64 bit patterns (thread: 16 columns of a row of x and of
-// a row of y): into colE, and that of column lane % 16 of the thread's half into *E.  Two passes: the largest exponent
+// a row of y): into colE, and that of column lane % 16 of the thread's half into *E, and whether it is zero.  Two passes: the largest exponent
 // of a column, then the sum of its squares scaled by it.  False (for all) if a column is out of range, or zero and
 // zero_ok is false.
 __device__ __forceinline__ bool column_exponents(const int64_t* cf, const int64_t* cq, int* colE, uint32_t* red, int* E,
-                                                 bool zero_ok = true) {
+                                                 bool* zero, bool zero_ok = true) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ch = threadIdx.x >> 8;
   uint32_t mymax = 0;
 #pragma unroll
@@ -187,6 +197,7 @@ __device__ __forceinline__ bool column_exponents(const int64_t* cf, const int64_
 #pragma unroll
   for (int q = 0; q < 8; ++q) s2 += __uint_as_float(red[(8 * ch + q) * 16 + (lane & 15)]);
   const int k = (int)(__float_as_uint(sqrtf(s2) * 1.03f) >> 23) - 127;
+  *zero = mx == 0;
   *E = mx == 0 ? 0 : k + 1 + emax - 1016;
   if ((warp & 7) == 0 && lane < 16) colE[16 * ch + lane] = *E;
   return true;
@@ -225,10 +236,67 @@ __device__ __forceinline__ void gram_partials(int64_t* P, uint32_t tq, int s) {
   }
 }
 
+// Bits of a warp's 32 rows, the CTA's two column halves in words warp and warp ^ 8: those of row r.
+__device__ __forceinline__ bool row_bit(const uint32_t* words) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  return ((words[warp] | words[warp ^ 8]) >> lane) & 1;
+}
+__device__ __forceinline__ uint32_t abs_hi(int64_t x) {        // upper word of |x| (of |x| - 1 for x < 0)
+  const int h = (int)(x >> 32);
+  return (uint32_t)(h ^ (h >> 31));
+}
+constexpr uint32_t kSmallRow = 1u << (31 - 8);                 // 2^-8 of a column, in the upper word of C
+
+// Whether the block would lose a row's own scale (see the head of this file).  Thread: row r of the strip, 16 columns;
+// big: its largest |C| (abs_hi), nz: V has an entry in the row, w2: rows 2 warp, 2 warp + 1 of W2 2^(62 - E_c) in column
+// lane, pivot: a pivot row is lost, diag: row of reflector 0's unit entry (out of range: in the pivot tile).  V's
+// digits and T are in place.  Called for few strips, outside the ordinary path's registers.
+__device__ __noinline__ bool rows_lost(unsigned char* sm, int kb, int eT, uint32_t big, bool nz, int64_t w20, int64_t w21,
+                                       bool pivot, bool narrow, int diag) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, r = tid & 255, ch = tid >> 8;
+  float* omega = reinterpret_cast<float*>(sm + kDigRow);       // max over c of |W2(j, c)| 2^-E_c
+  float* least = omega + 32;                                   // narrow: (2^-8 ||v_j||)^2 without the unit entry
+  uint32_t* bigs = reinterpret_cast<uint32_t*>(least + 32);
+  uint32_t* strong = bigs + 16;
+  const uint32_t h0 = __reduce_max_sync(kFull, abs_hi(w20)), h1 = __reduce_max_sync(kFull, abs_hi(w21));
+  const unsigned bm = __ballot_sync(kFull, big >= kSmallRow);
+  if (lane < 2) {
+    const int j = 2 * warp + lane;
+    omega[j] = (float)(lane ? h1 : h0) * 0x1p-30f;
+    const float tau = (float)reinterpret_cast<const int2*>(sm + kDigT)[35 * j].x * exp2f((float)(eT - 28));
+    least[j] = tau > 0.0f ? 0x1p-16f * fmaxf(2.0f / tau - 1.0f, 0x1p-12f) : 2.0f;      // ||v_j||^2 = 2 / tau_j
+  }
+  if (lane == 0) bigs[warp] = bm;
+  if (!__syncthreads_or((w20 | w21) != 0)) return __syncthreads_or(pivot) != 0;
+  const bool small = nz && !row_bit(bigs);
+  bool st = false;
+  if (__any_sync(kFull, small)) {
+    for (int g = 0; g < 2; ++g) {
+      // V(r, j) from its two upper digits (2^-14): |W2| is below 2 x 2^E_c
+      const unsigned char* o = sm + kDigV + r * 64 + (((2 * ch + g) ^ ((r >> 1) & 3)) << 4);
+      const uint4 a4 = *reinterpret_cast<const uint4*>(o), b4 = *reinterpret_cast<const uint4*>(o + kDigSlice);
+      const uint32_t a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        float hi, lo;
+        asm("cvt.f32.f16 %0, %1;" : "=f"(hi) : "h"((unsigned short)(a[q >> 1] >> (16 * (q & 1)))));
+        asm("cvt.f32.f16 %0, %1;" : "=f"(lo) : "h"((unsigned short)(b[q >> 1] >> (16 * (q & 1)))));
+        const float v = fabsf(fmaf(hi, 256.0f, lo)) * 0x1p-14f;
+        const int j = 16 * ch + 8 * g + q;
+        st = st || (j < kb && (v * omega[j] >= 0x1p-10f || (narrow && r != diag + j && v * v >= least[j])));
+      }
+    }
+  }
+  const unsigned sb = __ballot_sync(kFull, st);
+  if (lane == 0) strong[warp] = sb;
+  __syncthreads();
+  return __syncthreads_or(pivot || (small && !row_bit(strong))) != 0;
+}
+
 // Published blocks: what the updates of a reduction read of a panel block instead of V and T, made once by its factor
 // sub-task (a strip spent 4.4k of its 24k cycles a block on V's digits).  Digits of V in the operand layout
-// (digit_image_rows(nb) rows, zeros outside the block), T 2^(56 - eT) split as the updates read it, then two
-// integers: whether |v| <= 1 and eT <= 12 hold, and eT.
+// (digit_image_rows(nb) rows, zeros outside the block), T 2^(56 - eT) split as the updates read it, then the header: two
+// integers, whether |v| <= 1 and eT <= 12 hold, and eT, and from its word 4 on a bit for each row of V that is not zero.
 // Starts the copy of the V area (16 KB a digit) into block vd; wait_image before the sub-task ends.
 __device__ __forceinline__ void store_image(unsigned char* sm, unsigned char* vd, int nb) {
   if ((int)uniform(threadIdx.x >> 5) == kIssueWarp) {
@@ -247,12 +315,17 @@ __device__ __forceinline__ void wait_image() {
     asm volatile("fence.proxy.async;" ::: "memory");
   }
 }
-// T and the two integers; t: rows 2 warp, 2 warp + 1 of column lane, ok: the block's V is in range (any thread).
-__device__ __forceinline__ void publish_t(unsigned char* vd, int nb, const double* t, bool good, uint32_t* red) {
+// T and the header; t: rows 2 warp, 2 warp + 1 of column lane, good: the block's V is in range (any thread), nz: this
+// thread's half of row r of V has an entry.
+__device__ __forceinline__ void publish_t(unsigned char* vd, int nb, const double* t, bool good, bool nz, uint32_t* red) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t h = max((uint32_t)__double2hiint(t[0]) & 0x7fffffffu, (uint32_t)__double2hiint(t[1]) & 0x7fffffffu);
   const uint32_t hm = __reduce_max_sync(kFull, h);
-  if (lane == 0) red[warp] = hm;
+  const unsigned rows = __ballot_sync(kFull, nz);
+  if (lane == 0) {
+    red[warp] = hm;
+    red[16 + warp] = rows;
+  }
   const bool v_ok = __syncthreads_and(good ? 1 : 0) != 0;
   const int eT = max((int)(__reduce_max_sync(kFull, red[lane & 15]) >> 20) - 1022, 1);
   int2* Ts = reinterpret_cast<int2*>(vd + kDigN * digit_image_rows(nb) * 64);
@@ -262,15 +335,17 @@ __device__ __forceinline__ void publish_t(unsigned char* vd, int nb, const doubl
     const int x = (int)((f + (1 << 27)) >> 28);
     __stcg(Ts + (2 * warp + k) * 34 + lane, make_int2(x, (int)(f - ((int64_t)x << 28))));
   }
-  if (threadIdx.x == 0)
-    __stcg(reinterpret_cast<int2*>(vd + digit_block_bytes(nb) - 128), make_int2(v_ok && eT <= 12 ? 1 : 0, eT));
+  unsigned char* head = vd + digit_block_bytes(nb) - kDigitHeadBytes;
+  if (threadIdx.x == 0) __stcg(reinterpret_cast<int2*>(head), make_int2(v_ok && eT <= 12 ? 1 : 0, eT));
+  if (threadIdx.x < 8)
+    __stcg(reinterpret_cast<uint32_t*>(head) + 4 + threadIdx.x, red[16 + threadIdx.x] | red[24 + threadIdx.x]);
 }
 // Publishes a block that task_panel_factor has just written.
 __device__ __noinline__ void publish_block(unsigned char* sm, int kind, const double* X, int tr, const double* Tg, int nb,
                                            int ib, int b, unsigned char* vd) {
   const int tid = threadIdx.x, kb = ib, c0 = b * ib, r = tid & 255, cb = 16 * (tid >> 8);
   const int r0 = kind == PM_GE ? c0 : 0, r1 = kind == PM_TT ? c0 + kb : nb;
-  bool good = true;
+  bool good = true, nz = false;
   __syncthreads();
 #pragma unroll
   for (int g = 0; g < 2; ++g) {
@@ -284,6 +359,8 @@ __device__ __noinline__ void publish_block(unsigned char* sm, int kind, const do
         if (kind == PM_GE && d == 0) x = 1.0;
       }
       good = good && ((uint32_t)__double2hiint(x) & 0x7fffffffu) <= 0x3ff00000u;
+      if (((uint32_t)__double2hiint(x) & 0x7fffffffu) != 0)      // (not the unit entry of H = I)
+        nz = nz || kind != PM_GE || d != 0 || ldg(Tg + (size_t)c0 * ib + c * (kb + 1)) != 0.0;
       v[a] = to_fixed(x, 62);
     }
     put_digits(sm + kDigV, r, (cb >> 3) + g, v);
@@ -295,7 +372,7 @@ __device__ __noinline__ void publish_block(unsigned char* sm, int kind, const do
   double t[2];
 #pragma unroll
   for (int k = 0; k < 2; ++k) t[k] = (arow + k < kb && lane < kb) ? ldg(Tg + (size_t)c0 * ib + arow + k + lane * kb) : 0.0;
-  publish_t(vd, nb, t, good, reinterpret_cast<uint32_t*>(sm + kDigHead + 128));
+  publish_t(vd, nb, t, good, nz, reinterpret_cast<uint32_t*>(sm + kDigHead + 128));
   wait_image();
   __syncthreads();
 }
@@ -336,7 +413,7 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
     if (lane < kDigN) bulk_copy(sm + kDigV + lane * kDigSlice + o, src + lane * img + o, size, um.mbar + 24);
   };
   auto load_head = [&](int b) {
-    return __ldcg(reinterpret_cast<const int2*>(vd + (size_t)(b + 1) * digit_block_bytes(nb) - 128));
+    return __ldcg(reinterpret_cast<const int2*>(vd + (size_t)(b + 1) * digit_block_bytes(nb) - kDigitHeadBytes));
   };
   int2 head = make_int2(1, 0);       // published block: whether it is in range, exponent of T
   // V block of the next application, as stored, into the staging area: columns (ld 256) for tr = 0, by bulk copies
@@ -418,13 +495,24 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
     int64_t cq[16];
     load_row(Cp, ownp, cq);
     int E;
-    if (!column_exponents(cf, cq, colE, red, &E)) {
+    bool zero;
+    if (!column_exponents(cf, cq, colE, red, &E, &zero)) {
       wait_v();
       __syncthreads();
       return 0;
     }
+    uint32_t big = 0;
 #pragma unroll
-    for (int c = 0; c < 16; ++c) cf[c] = to_fixed(__longlong_as_double(cf[c]), 63 - __shfl_sync(kFull, E, c));
+    for (int c = 0; c < 16; ++c) {
+      cf[c] = to_fixed(__longlong_as_double(cf[c]), 63 - __shfl_sync(kFull, E, c));
+      big = max(big, abs_hi(cf[c]));
+    }
+    uint32_t* rw = reinterpret_cast<uint32_t*>(sm + kDigRow);
+    const unsigned rows = __ballot_sync(kFull, big >= kSmallRow), cols = __ballot_sync(kFull, !zero && lane < 16);
+    if (lane == 0) {
+      rw[warp] = rows;
+      if ((warp & 7) == 0) rw[16 + ch] = __popc(cols);
+    }
   }
 
   const uint32_t uV = uniform(smem_u32(sm + kDigV)), uC = uV + kDigC, uW = uV + kDigW2, utm = uniform(um.tmem);
@@ -432,6 +520,10 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
   int done = 0, v0 = 0, v1 = 0, c0 = 0;
   __syncthreads();
   const int myE = colE[lane];          // of column c = lane (the pivot rows' column)
+  const uint32_t* rw = reinterpret_cast<const uint32_t*>(sm + kDigRow);
+  const int ncols_nz = (int)(rw[16] + rw[17]);         // columns that are not zero
+  const bool small_row = ncols_nz > 0 && !row_bit(rw);
+  bool touched = false;                // a reflector applied so far has an entry in row r
   bool ok = true;                      // this thread's completion waits
   for (int bb = 0; bb < nbk; ++bb) {
     // ---- V digits ---------------------------------------------------------------------------------
@@ -491,7 +583,11 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
         }
         uint32_t ht = max((uint32_t)__double2hiint(tv[0]) & 0x7fffffffu, (uint32_t)__double2hiint(tv[1]) & 0x7fffffffu);
         ht = __reduce_max_sync(kFull, ht);
-        if (lane == 0) red[warp] = ht;
+        const unsigned rows = __ballot_sync(kFull, hv != 0);
+        if (lane == 0) {
+          red[warp] = ht;
+          red[16 + warp] = rows;
+        }
       }
       // the staged V is free from here on: the C digits take its place.  1: a wait ran out, 2: |v| > 1 (not finite)
       if (__syncthreads_or(!ok || hv > 0x3ff00000u)) {
@@ -532,8 +628,9 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
     int2* Ts = reinterpret_cast<int2*>(sm + kDigT);       // op(T)(a, t) at t 34 + a: 2^28 x + y = T 2^(56 - eT)
     if constexpr (kPre) {
       if (uwarp == kIssueWarp && lane == 0) {
-        mbar_expect(um.mbar + 32, kDigTBytes);
-        bulk_copy(Ts, vd + (size_t)blk_of(bb) * digit_block_bytes(nb) + kDigN * img, kDigTBytes, um.mbar + 32);
+        mbar_expect(um.mbar + 32, kDigTBytes + kDigitHeadBytes);
+        bulk_copy(Ts, vd + (size_t)blk_of(bb) * digit_block_bytes(nb) + kDigN * img, kDigTBytes + kDigitHeadBytes,
+                  um.mbar + 32);
       }
       if (bb + 1 < nbk) {
         head = load_head(blk_of(bb + 1));
@@ -612,9 +709,38 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
 #pragma unroll
       for (int i = 0; i < 8; ++i) *reinterpret_cast<uint32_t*>(p + i * 2048) = d[i];
     }
+    // ---- rows that fixed point would lose ------------------------------------------------------------
+    bool nz, pivot = false;            // V has an entry in row r; a pivot row is lost
+    if constexpr (kPre) {
+      nz = (reinterpret_cast<const uint32_t*>(sm + kDigT + kDigTBytes)[4 + (warp & 7)] >> lane) & 1;
+    } else {
+      nz = row_bit(red + 16);
+      if (type == UNMQR && r >= c0 && r < c0 + kb && Ts[35 * (r - c0)].x == 0) {      // (not the unit entry of H = I)
+        nz = false;
+        for (int a = c0; a < r; ++a) nz = nz || ldg(X + toff(r, a, nb, tr)) != 0.0;
+      }
+    }
+    if (top) {
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        if (Ts[(arow + k) * 35].x > ((1 << 29) - (1 << 14)) >> eT) {      // tau, warp-uniform
+          const bool is_big = __any_sync(kFull, abs_hi(c63[k]) >= kSmallRow || abs_hi(w2[k]) >= 1u << (30 - 10));
+          pivot = pivot || (__any_sync(kFull, w2[k] != 0) && !is_big);
+        }
+    }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
+    if (__syncthreads_or(pivot || (small_row && nz))) {
+      uint32_t big = 0;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) big = max(big, abs_hi(cf[c]));
+      // uniform: the rest goes to the FP64 units
+      if (rows_lost(sm, kb, eT, big, nz, w2[0], w2[1], pivot, ncols_nz < 8, type == UNMQR ? c0 : -kDigRows)) {
+        if (!kPre && bb + 1 < nbk) ok = wait_v() && ok;
+        break;
+      }
+    }
+    touched = touched || nz;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     // ---- phase 3: V W2, digit pairs of equal weight in one accumulator ------------------------------
     if (uwarp == kIssueWarp) {
@@ -632,7 +758,7 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
     }
 #pragma unroll
     for (int k = 0; k < 2; ++k)
-      if (top && lane < ncols && arow + k < kb)
+      if (top && lane < ncols && arow + k < kb && w2[k] != 0)
         stg(Cp + toff(c0 + arow + k, col0 + lane, nb, tr), from_fixed(c63[k] - 2 * w2[k], 63 - myE));
     // ---- C -= V W2 in integers: C 2^(63 - E_c) loses D_g 2^(51 - 8 g) -------------------------------
     if (kPre && uwarp == kIssueWarp && bb + 1 < nbk) {
@@ -676,7 +802,7 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
     return nbk;
   }
   // ---- store the strip ----------------------------------------------------------------------------
-  if (own && done > 0) {
+  if (own && touched) {
     if (tr) {
 #pragma unroll
       for (int c = 0; c < 16; c += 2)
