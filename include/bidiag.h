@@ -66,7 +66,9 @@ enum {
   BIDIAG_OPT_DEBUG_UNSET_DEP = 3, /* 1: the next bidiag_band adds to its first task a dependency on a
                                      flag nothing sets, so that its wait runs out (failure-path test) */
   BIDIAG_OPT_STRIP = 4,           /* column-strip width of the update tasks (16, 32 or 64; default 32, and
-                                     64 for a one-matrix reduction with FP32 storage) */
+                                     64 for a one-matrix reduction with FP32 storage).  FP64 matrices whose
+                                     strips come out wider than 32 columns run wholly on the FP64 units, which
+                                     is several times slower from tiles of 64 on */
   BIDIAG_OPT_TIMING = 5,          /* 1: time the executor launch of each bidiag_band with CUDA events */
   BIDIAG_OPT_TRACE = 6,           /* 1: record a per-task trace of each bidiag_band (see bidiag_trace) */
   BIDIAG_OPT_F32_UPDATES = 7,     /* FP32 storage: 0 = updates as three TF32 tensor-core products, the

@@ -849,7 +849,7 @@ int band_batched_impl(bidiag_handle h, int64_t count, const int64_t* m, const in
     mi.w = pl.strip_w;
     mi.npanels = pl.npanels;
     mi.offV = bp->totV;
-    if (esize == 8 && bd::digits_fit(pl.nb, pl.ib, pl.ib))
+    if (esize == 8 && bd::digits_tmem(pl.nb, pl.ib, pl.strip_w) > 0)
       bp->totV += (int64_t)pl.npanels * (pl.nb / pl.ib) * bd::digit_block_bytes(pl.nb);
     bp->tiles_all += mi.ntiles[0];
     bp->cols_all += n[b];

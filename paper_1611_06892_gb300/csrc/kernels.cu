@@ -704,11 +704,12 @@ __device__ __forceinline__ void inverse32(const double* G, const double* d, doub
 // T[l,l] = tau_l, T[0:l, l] = -tau_l T[0:l, 0:l] G[0:l, l] inside diagonal blocks of 8 columns (all blocks at once),
 // then blocks are merged pairwise, [T11 T12; 0 T22] with T12 = -T11 G12 T22 (the product of two compact WY blocks),
 // so the sequential depth is 8 + 2 log2(kb/8) barrier steps instead of kb.
+// fixed32: by inverse32 (digit executor, kb = ldt = 32).
 template <typename E>
-__device__ void t_from_gram(int kb, const double* tau_s, E* Tb, int ldt, E* G) {
+__device__ void t_from_gram(int kb, const double* tau_s, E* Tb, int ldt, E* G, bool fixed32) {
   E* Y = G + kb * kb;
 #if BD_EXEC_PART == 1
-  if (kb == 32 && ldt == 32) {
+  if (fixed32) {
     inverse32(G, tau_s, Tb, Y);
     return;
   }
@@ -763,7 +764,7 @@ __device__ void t_from_gram(int kb, const double* tau_s, E* Tb, int ldt, E* G) {
 // blocks per thread (no cross-lane reductions).
 template <typename E>
 __device__ void build_t(int mode, const E* P, int lp, int rows, int kb, int voff, const double* tau_s, E* Tb, int ldt,
-                        E* G) {
+                        E* G, bool fixed32) {
   // reflector tail values: GE unit lower trapezoid, TS the full tail, TT the tail up to row voff + c
   auto vval = [&](int r, int c) -> E {
     if (mode == PM_GE) return r > c ? P[r + c * lp] : (r == c ? E(1) : E(0));
@@ -808,7 +809,7 @@ __device__ void build_t(int mode, const E* P, int lp, int rows, int kb, int voff
     if (a1 < l1 && a1 != a0 && l1 != l0) G[a1 + l1 * kb] = s11;
   }
   __syncthreads();
-  t_from_gram(kb, tau_s, Tb, ldt, G);
+  t_from_gram(kb, tau_s, Tb, ldt, G, fixed32);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1336,7 +1337,7 @@ __device__ bool apply_rm_umma(const float* Vh, const float* Vl, int vrows, int k
 // ---------------------------------------------------------------------------------------------
 template <typename E>
 __device__ void task_panel_factor(unsigned char* smb, int kind, E* X, E* A, int tr, E* Tg, int nb, int ib, int b,
-                                  bool pair_scalars) {
+                                  bool pair_scalars, bool fixed32 = false) {
   const Layout L = layout_panel(nb, ib, (int)sizeof(E));
   double* tau = reinterpret_cast<double*>(smb);
   double* red = tau + 64;
@@ -1348,7 +1349,7 @@ __device__ void task_panel_factor(unsigned char* smb, int kind, E* X, E* A, int 
     load_tile(P, 1, L.lp, X, nb, tr, c0, c0, rows, kb, M_NONE);
     __syncthreads();
     factor_panel(PM_GE, P, L.lp, rows, kb, (E*)nullptr, 0, 0, tau, red, pair_scalars);
-    build_t(PM_GE, P, L.lp, rows, kb, 0, tau, Tb, kb, G);
+    build_t(PM_GE, P, L.lp, rows, kb, 0, tau, Tb, kb, G, fixed32);
     store_tile(P, 1, L.lp, X, nb, tr, c0, c0, rows, kb, M_NONE);
   } else {
     const bool tt = kind == PM_TT;
@@ -1357,7 +1358,7 @@ __device__ void task_panel_factor(unsigned char* smb, int kind, E* X, E* A, int 
     load_tile(P, 1, L.lp, X, nb, tr, 0, c0, vrows, kb, tt ? M_UPPER : M_NONE);
     __syncthreads();
     factor_panel(kind, P, L.lp, vrows, kb, Rt, kb, c0, tau, red, pair_scalars);
-    build_t(kind, P, L.lp, vrows, kb, c0, tau, Tb, kb, G);
+    build_t(kind, P, L.lp, vrows, kb, c0, tau, Tb, kb, G, fixed32);
     store_tile(Rt, 1, kb, A, nb, tr, c0, c0, kb, kb, M_UPPER);
     store_tile(P, 1, L.lp, X, nb, tr, 0, c0, vrows, kb, tt ? M_UPPER : M_NONE);
   }
@@ -1611,10 +1612,10 @@ __device__ bool task_update_umma(unsigned char* smb, int type, const float* X, f
 #include "panel_digits.cuh"
 
 // An update (strip or panel block, arguments as task_update) on the tensor cores where the CTA holds TMEM for it
-// and the sizes fit, on the FMA units otherwise; true if any of it ran on tcgen05.
+// and the sizes fit (FP64: dig), on the FMA units otherwise; true if any of it ran on tcgen05.
 template <typename E, bool kDig>
 __device__ __forceinline__ bool run_update(unsigned char* smb, int type, const E* X, E* Cp, E* C, int tr, bool notrans, const E* Tg,
-                           int nb, int ib, int w, int blk0, int blk1, int col0, int ncols, const unsigned char* vd,
+                           int nb, int ib, int w, int blk0, int blk1, int col0, int ncols, bool dig, const unsigned char* vd,
                            Umma& um, const ExecParams& prm) {
   int done = 0;
   if constexpr (sizeof(E) == 4) {
@@ -1624,7 +1625,7 @@ __device__ __forceinline__ bool run_update(unsigned char* smb, int type, const E
   }
 #if BD_EXEC_PART == 1
   if constexpr (kDig) {
-    if (um.ncols_alloc >= kDigTmem && digits_fit(nb, ib, ncols))
+    if (dig)
       done = vd ? task_update_digits<true>(smb, type, X, Cp, C, tr, notrans, Tg, nb, ib, blk0, blk1, col0, ncols, vd, um, prm)
                 : task_update_digits<false>(smb, type, X, Cp, C, tr, notrans, Tg, nb, ib, blk0, blk1, col0, ncols, vd, um, prm);
     if (done == blk1 - blk0) return true;
@@ -2249,10 +2250,13 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
                 ? static_cast<E*>(prm.T) + mv.offT + (size_t)t.tslot * ib * nb
                 : nullptr;
     if constexpr (!kBwd) {
-    // published blocks of this sub-task's panel (Q^T programs of the digit instantiation)
+    // Digit products: one answer for all sub-tasks of a matrix, from its own sizes and strip width, so that a matrix of
+    // a batch gets the bits it gets alone; published blocks of this sub-task's panel (Q^T programs)
+    bool dig = false;
     unsigned char* vd = nullptr;
     if constexpr (kDig) {
-      if (prm.vd && Tg && !notrans && digits_fit(nb, ib, ib))
+      dig = um.ncols_alloc >= kDigTmem && digits_fit(nb, ib, min(wst, nb));
+      if (prm.vd && Tg && !notrans && dig)
         vd = prm.vd + mv.offV + (int64_t)t.tslot * nblk * digit_block_bytes(nb);
     }
     switch (type) {
@@ -2260,11 +2264,11 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
         E* A = (kind == PM_GE) ? nullptr : tile_ptr<E>(prm, mv, t.a, ok);
         if (ok && Tg && blk < nblk && kind <= PM_TT) {
 #if BD_EXEC_PART == 1
-          if (um.ncols_alloc >= kDigTmem && digits_fit(nb, ib, ib))
+          if (dig)
             on_tc5 = task_panel_digits(smb, kind, X, A, tr, Tg, nb, ib, blk,
                                        vd ? vd + blk * digit_block_bytes(nb) : nullptr, um, prm);
           if (!on_tc5) {
-            task_panel_factor(smb, kind, X, A, tr, Tg, nb, ib, blk, false);
+            task_panel_factor(smb, kind, X, A, tr, Tg, nb, ib, blk, false, dig && ib == 32);
             if (vd) publish_block(smb, kind, X, tr, Tg, nb, ib, blk, vd + blk * digit_block_bytes(nb));
           }
 #else
@@ -2279,8 +2283,8 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
         E* A = (kind == PM_GE) ? nullptr : tile_ptr<E>(prm, mv, t.a, ok);
         const int utype = kind == PM_GE ? UNMQR : (kind == PM_TS ? TSMQR : TTMQR);
         if (ok && Tg && blk < strip && strip < nblk && kind <= PM_TT)
-          on_tc5 = run_update<E, kDig>(smb, utype, X, A, X, tr, false, Tg, nb, ib, wst, blk, blk + 1, strip * ib, ib, vd, um,
-                                       prm);
+          on_tc5 = run_update<E, kDig>(smb, utype, X, A, X, tr, false, Tg, nb, ib, wst, blk, blk + 1, strip * ib, ib, dig, vd,
+                                       um, prm);
         else
           ok = false;
         break;
@@ -2292,8 +2296,8 @@ __global__ void __launch_bounds__(kThreads, 1) exec_kernel(const ExecParams prm)
         E* C = tile_ptr<E>(prm, mv, t.c, ok);
         const int col0 = strip * wst;
         if (ok && Tg && col0 < nb)
-          on_tc5 = run_update<E, kDig>(smb, type, X, A, C, tr, notrans, Tg, nb, ib, wst, 0, nblk, col0, min(wst, nb - col0), vd,
-                                       um, prm);
+          on_tc5 = run_update<E, kDig>(smb, type, X, A, C, tr, notrans, Tg, nb, ib, wst, 0, nblk, col0, min(wst, nb - col0), dig,
+                                       vd, um, prm);
         else
           ok = false;
         break;
