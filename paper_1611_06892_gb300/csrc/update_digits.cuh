@@ -445,6 +445,16 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
     um.phase ^= 8u;
     return w;
   };
+  // A completion wait ran out (for any thread): the error word is set, nothing more is issued or written back, the copies
+  // and MMAs in flight are waited for (with the same limit)
+  auto timed_out = [&]() {
+    if (tid == 0) atomicCAS(prm.err, 0, DERR_TIMEOUT);
+    for (int b = 0; b < 5; ++b) mbar_wait(um.mbar + 8 * b, ((um.phase >> b) & 1u) ^ 1u, prm.wait_ns);
+    for (int b = 3; b < 5; ++b) mbar_wait(um.mbar + 8 * b, (um.phase >> b) & 1u, prm.wait_ns);
+    cp_async_wait_all();
+    __syncthreads();
+    return nbk;
+  };
   // T of a block: entries tid + 512 k of the kb x kb block as stored
   double tv[2];
   auto load_t = [&](int c0) {
@@ -497,9 +507,8 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
     int E;
     bool zero;
     if (!column_exponents(cf, cq, colE, red, &E, &zero)) {
-      wait_v();
-      __syncthreads();
-      return 0;
+      // (the caller's next update writes where the copy of V lands)
+      return __syncthreads_and(wait_v() ? 1 : 0) ? 0 : timed_out();
     }
     uint32_t big = 0;
 #pragma unroll
@@ -537,7 +546,7 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
         break;
       }
       if (!head.x) {                                // uniform: the rest goes to the FP64 units
-        wait_v();
+        ok = wait_v() && ok;
         break;
       }
       eT = head.y;
@@ -791,16 +800,7 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
     for (int h = h0; h < h1; ++h) um.phase ^= 2u << h;
     ++done;
   }
-  // a completion wait ran out (the error word is set): nothing more is issued or written back, the copies and MMAs
-  // in flight are waited for (with the same limit)
-  if (!__syncthreads_and(ok ? 1 : 0)) {
-    if (tid == 0) atomicCAS(prm.err, 0, DERR_TIMEOUT);
-    for (int b = 0; b < 5; ++b) mbar_wait(um.mbar + 8 * b, ((um.phase >> b) & 1u) ^ 1u, prm.wait_ns);
-    for (int b = 3; b < 5; ++b) mbar_wait(um.mbar + 8 * b, (um.phase >> b) & 1u, prm.wait_ns);
-    cp_async_wait_all();
-    __syncthreads();
-    return nbk;
-  }
+  if (!__syncthreads_and(ok ? 1 : 0)) return timed_out();
   // ---- store the strip ----------------------------------------------------------------------------
   if (own && touched) {
     if (tr) {
