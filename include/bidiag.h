@@ -127,7 +127,10 @@ typedef struct bidiag_reflectors {
 } bidiag_reflectors;
 
 /* Creates a handle bound to CUDA device `device` and stream `cuda_stream` (a cudaStream_t; NULL =
- * the legacy default stream).  Owns the plan cache and the scheduler workspace.
+ * the legacy default stream).  Owns the plan cache, the scheduler workspace and, from its first FP64 reduction on the
+ * tensor cores on, up to 2 GiB of device memory for the factors' digits (npanels nb / ib blocks of 120 KB at nb 256:
+ * 1.15 GB for 8192^2 Auto; larger ones are allocated per call).  bidiag_destroy gives it back, and so does the handle
+ * when an allocation of its own would fail.
  * Errors: -1 (h NULL), -2 (bad device), BIDIAG_ERR_CUDA, BIDIAG_ERR_NOMEM. */
 int bidiag_create(bidiag_handle* h, int device, void* cuda_stream);
 

@@ -155,6 +155,30 @@ int cuda_fail(bidiag_handle h, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail(h, e_, #call); \
   } while (0)
 
+// Gives the kept storage of published blocks back (its memory returns to the device at the synchronisation).
+void release_vd(bidiag_handle h) {
+  if (!h->d_vd) return;
+  cudaFreeAsync(h->d_vd, h->stream);
+  h->d_vd = nullptr;
+  h->vd_cap = 0;
+  cudaStreamSynchronize(h->stream);
+}
+
+// alloc(), once more without that storage when the device is out of memory.
+template <typename F>
+cudaError_t with_memory(bidiag_handle h, F alloc) {
+  cudaError_t e = alloc();
+  if (e == cudaErrorMemoryAllocation && h->d_vd) {
+    cudaGetLastError();
+    release_vd(h);
+    e = alloc();
+  }
+  return e;
+}
+cudaError_t dev_malloc(bidiag_handle h, void** p, size_t bytes) {
+  return with_memory(h, [&] { return cudaMalloc(p, bytes); });
+}
+
 void dump_tasks(const std::vector<bd::Task>& tasks, std::vector<int32_t>& out) {
   out.resize(tasks.size() * 6);
   for (size_t x = 0; x < tasks.size(); ++x) {
@@ -169,9 +193,9 @@ int upload_program(bidiag_handle h, PlanDev& pd, const std::vector<bd::DevTask>&
   const size_t nt = dev.size();
   pd.nflags = (int)nt + extra_flags;
   pd.ndeps = (int64_t)deps.size();
-  CK(h, cudaMalloc(&pd.d_tasks, std::max<size_t>(1, nt) * sizeof(bd::DevTask)));
-  CK(h, cudaMalloc(&pd.d_deps, std::max<size_t>(1, deps.size()) * sizeof(int32_t)));
-  CK(h, cudaMalloc(&pd.d_done, std::max<size_t>(1, pd.nflags) * sizeof(int)));
+  CK(h, dev_malloc(h, (void**)&pd.d_tasks, std::max<size_t>(1, nt) * sizeof(bd::DevTask)));
+  CK(h, dev_malloc(h, (void**)&pd.d_deps, std::max<size_t>(1, deps.size()) * sizeof(int32_t)));
+  CK(h, dev_malloc(h, (void**)&pd.d_done, std::max<size_t>(1, pd.nflags) * sizeof(int)));
   if (nt) CK(h, cudaMemcpy(pd.d_tasks, dev.data(), nt * sizeof(bd::DevTask), cudaMemcpyHostToDevice));
   if (!deps.empty()) CK(h, cudaMemcpy(pd.d_deps, deps.data(), deps.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
   return BIDIAG_OK;
@@ -257,7 +281,7 @@ int run_exec(bidiag_handle h, const PlanDev& pd, int ntasks, void* b0, int64_t n
     if (h->trace_cap < ntasks) {
       if (h->d_trace) CK(h, cudaFree(h->d_trace));
       h->d_trace = nullptr;
-      CK(h, cudaMalloc(&h->d_trace, sizeof(int64_t) * 4 * (size_t)ntasks));
+      CK(h, dev_malloc(h, (void**)&h->d_trace, sizeof(int64_t) * 4 * (size_t)ntasks));
       h->trace_cap = ntasks;
     }
     prm.trace = h->d_trace;
@@ -272,8 +296,9 @@ int run_exec(bidiag_handle h, const PlanDev& pd, int ntasks, void* b0, int64_t n
   CK(h, cudaMemsetAsync(pd.d_done, 0, sizeof(int) * (size_t)pd.nflags, h->stream));
   CK(h, cudaMemsetAsync(h->d_ctrl, 0, sizeof(int), h->stream));
   // published panel blocks live for the launch only.  Up to kVdKeep bytes of storage stay with the handle, whose
-  // launches are ordered on its stream (8192^2: 1.6 GB, 3 ms to map when the pool had been trimmed at a
-  // synchronisation); without memory for them the updates do without
+  // launches are ordered on its stream (8192^2 Auto: 1.15 GB, 3 ms to map when the pool had been trimmed at a
+  // synchronisation), until it is destroyed or an allocation of its own fails (with_memory); without memory for them
+  // the updates do without
   const bool vd_kept = vd_bytes <= kVdKeep;
   if (digits && vd_bytes > 0) {
     if (vd_kept && h->vd_cap >= vd_bytes) {
@@ -367,7 +392,7 @@ template <typename T>
 int dev_alloc(bidiag_handle h, T** p, size_t count) {
   *p = nullptr;
   if (count == 0) return BIDIAG_OK;
-  cudaError_t e = cudaMallocAsync((void**)p, count * sizeof(T), h->stream);
+  cudaError_t e = with_memory(h, [&] { return cudaMallocAsync((void**)p, count * sizeof(T), h->stream); });
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaMallocAsync");
   return BIDIAG_OK;
 }
@@ -604,8 +629,8 @@ int adjoint_setup(bidiag_handle h, bidiag_result_t r, int esize, AdjointSizes* z
     }
     int rc = upload_program(h, bw->prog, bw->bp.dev, bw->bp.deps, 1);
     if (rc) return rc;
-    CK(h, cudaMalloc(&bw->d_slot_off, bw->bp.slot_off.size() * sizeof(int64_t)));
-    CK(h, cudaMalloc(&bw->d_pinfo, bw->bp.pinfo.size() * sizeof(int32_t)));
+    CK(h, dev_malloc(h, (void**)&bw->d_slot_off, bw->bp.slot_off.size() * sizeof(int64_t)));
+    CK(h, dev_malloc(h, (void**)&bw->d_pinfo, bw->bp.pinfo.size() * sizeof(int32_t)));
     CK(h, cudaMemcpy(bw->d_slot_off, bw->bp.slot_off.data(), bw->bp.slot_off.size() * sizeof(int64_t),
                      cudaMemcpyHostToDevice));
     CK(h, cudaMemcpy(bw->d_pinfo, bw->bp.pinfo.data(), bw->bp.pinfo.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
@@ -866,7 +891,7 @@ int band_batched_impl(bidiag_handle h, int64_t count, const int64_t* m, const in
   int rc0 = upload_program(h, bp->prog, dev, deps, 1);
   if (rc0) return rc0;
   bp->ntasks = (int)dev.size();
-  CK(h, cudaMalloc(&bp->d_mats, sizeof(bd::MatInfo) * (size_t)count));
+  CK(h, dev_malloc(h, (void**)&bp->d_mats, sizeof(bd::MatInfo) * (size_t)count));
   CK(h, cudaMemcpy(bp->d_mats, bp->info.data(), sizeof(bd::MatInfo) * (size_t)count, cudaMemcpyHostToDevice));
   if (h->batches.size() >= 8) h->batches.clear();
   h->batches[key] = bp;
@@ -878,10 +903,10 @@ int band_batched_impl(bidiag_handle h, int64_t count, const int64_t* m, const in
   auto store = std::make_shared<BatchStore>();
   store->plan = bp;
   int rc = 0;
-  CK(h, cudaMalloc(&store->tiles, (size_t)std::max<int64_t>(1, tot0) * esize));
-  if (tot1) CK(h, cudaMalloc(&store->tiles2, (size_t)tot1 * esize));
-  CK(h, cudaMalloc(&store->T, (size_t)std::max<int64_t>(1, totT) * esize));
-  CK(h, cudaMalloc(&store->d_desc, sizeof(bd::PackDesc) * 2 * (size_t)count));
+  CK(h, dev_malloc(h, (void**)&store->tiles, (size_t)std::max<int64_t>(1, tot0) * esize));
+  if (tot1) CK(h, dev_malloc(h, (void**)&store->tiles2, (size_t)tot1 * esize));
+  CK(h, dev_malloc(h, (void**)&store->T, (size_t)std::max<int64_t>(1, totT) * esize));
+  CK(h, dev_malloc(h, (void**)&store->d_desc, sizeof(bd::PackDesc) * 2 * (size_t)count));
   // results and their bands
   std::vector<bidiag_result*> res((size_t)count, nullptr);
   auto bail = [&](int code) {
