@@ -531,7 +531,21 @@ const AutotuneRow kAutotuneTable[] = {
 //    to ib).
 // Mode 0 is the flop count alone, with FP32-storage panel factors counted twice.
 enum WeightClass { W_PF_GE, W_PF_TS, W_PF_TT, W_PU_GE, W_PU_TS, W_PU_TT, W_UNMQR, W_TSMQR, W_TTMQR };
-static int64_t sub_time(int64_t flops, int cls, int64_t rows, int nb, int ib, int esize, int mode, bool digits) {
+static const AutotuneRow* nearest_row(int nb, int ib, int esize) {
+  const AutotuneRow* best = nullptr;
+  double dist = 0.0;
+  for (const AutotuneRow* r = kAutotuneTable; r->esize; ++r) {
+    const double d = std::fabs(std::log2((double)nb / r->nb)) + std::fabs(std::log2((double)ib / r->ib));
+    if (r->esize == esize && (!best || d < dist)) {
+      best = r;
+      dist = d;
+    }
+  }
+  return best;
+}
+// (best: nearest_row of these sizes, looked up once a plan: a third of the planning of 300 x 200 with tiles of 32 otherwise)
+static int64_t sub_time(int64_t flops, int cls, int64_t rows, int nb, int ib, int esize, int mode, bool digits,
+                        const AutotuneRow* best) {
   static const int64_t kDig[9] = {6700, 5900, 5500, 2250, 2500, 2100, 1180, 1380, 1220};
   static const int64_t kF32Base[6] = {4000, 3700, 4500, 500, 600, 550}, kF32Row[6] = {17, 12, 14, 2, 2, 2};
   static const int64_t kF32[3] = {576, 453, 650};   // per Mflop
@@ -541,15 +555,6 @@ static int64_t sub_time(int64_t flops, int cls, int64_t rows, int nb, int ib, in
   if (esize == 4 && ib == 32 && nb >= 96) {
     if (cls < W_UNMQR) return kDispatch + kF32Base[cls] + kF32Row[cls] * rows;
     return kDispatch + 1400 + flops * kF32[cls - W_UNMQR] / 1000000;
-  }
-  const AutotuneRow* best = nullptr;
-  double dist = 0.0;
-  for (const AutotuneRow* r = kAutotuneTable; r->esize; ++r) {
-    const double d = std::fabs(std::log2((double)nb / r->nb)) + std::fabs(std::log2((double)ib / r->ib));
-    if (r->esize == esize && (!best || d < dist)) {
-      best = r;
-      dist = d;
-    }
   }
   double us = best->us[cls];
   if (cls <= W_PF_TT) {
@@ -673,6 +678,7 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
   std::vector<int64_t> rd, wr;
   const int64_t ib2 = (int64_t)ib * ib;
   const bool digits = esize == 8 && digits_fit(nb, ib, w);
+  const AutotuneRow* row = nearest_row(nb, ib, esize);
 
   auto tref = [&](int buf, int oa, int ob, bool lq) {
     const int x = lq ? ob : oa, y = lq ? oa : ob;
@@ -713,7 +719,7 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
         wr.push_back(it.t(slot, b));
         const int64_t rows = kind == PK_GE ? nb - (int64_t)b * ib : (kind == PK_TS ? nb : (int64_t)(b + 1) * ib);
         d.op = make_op(PF, lq, false, 0, b, kind);
-        last = g.add(d, sub_time(12 * ib2 * rows, W_PF_GE + kind, rows, nb, ib, esize, prio, digits), rd, wr, -1);
+        last = g.add(d, sub_time(12 * ib2 * rows, W_PF_GE + kind, rows, nb, ib, esize, prio, digits, row), rd, wr, -1);
         // PU(b, s)
         for (int s = b + 1; s < nblk; ++s) {
           rd.clear();
@@ -734,7 +740,7 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
           }
           rd.push_back(it.t(slot, b));
           d.op = make_op(PU, lq, false, s, b, kind);
-          last = g.add(d, sub_time(6 * ib2 * rows, W_PU_GE + kind, rows, nb, ib, esize, prio, digits), rd, wr, -1);
+          last = g.add(d, sub_time(6 * ib2 * rows, W_PU_GE + kind, rows, nb, ib, esize, prio, digits, row), rd, wr, -1);
         }
       }
       panel_last[x] = last;
@@ -760,7 +766,7 @@ void build_plan(Plan& pl, int64_t m, int64_t n, int nb, int ib, int tree, int va
         }
         d.op = make_op(t.type, lq, false, s, 0, 0);
         g.add(d, sub_time(per_strip, t.type == UNMQR ? W_UNMQR : (t.type == TSMQR ? W_TSMQR : W_TTMQR), nb, nb, ib,
-                          esize, prio, digits),
+                          esize, prio, digits, row),
               rd, wr, panel_last[owner]);
       }
     } else {   // COPY(i, j): R part of A's tile (i, j) into the second phase's tile (i, j)
