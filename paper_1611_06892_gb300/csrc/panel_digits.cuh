@@ -428,7 +428,7 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
       cf[c] = cb + c < ti ? min(max((int64_t)__mul64hi(Bs[ti * 33 + cb + c] << 2, dinv[cb + c] << 2) << 4, -one), one)
                           : (cb + c == ti ? one + 1 : 0);
   }
-  bool nz = false;                     // V has an entry in the thread's half row
+  bool nz = false, strong = false;     // V has an entry in the thread's half row, one of 2^-8 beside the unit entry
   if (own && ok) {
 #pragma unroll
     for (int c = 0; c < 16; c += 2) {
@@ -436,7 +436,8 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
       const bool on = cb + c < kb, w0 = on && (ge ? d > 0 : (!tt || d <= 0)), w1 = on && (ge ? d > 1 : (!tt || d <= 1));
       double* p = X + toff(r, c0 + cb + c, nb, tr);
       const double x = from_fixed(cf[c], 62), y = from_fixed(cf[c + 1], 62);
-      nz = nz || x != 0.0 || y != 0.0;
+      nz = nz || (abs_hi(x) | abs_hi(y)) != 0;
+      strong = strong || (abs_hi(x) >= kStrong && !(ge && d == 0)) || (abs_hi(y) >= kStrong && !(ge && d == 1));
       cf[c] = to_fixed(x, 62);                            // V as it is stored
       cf[c + 1] = to_fixed(y, 62);
       if (tr && w0 && w1) {
@@ -468,7 +469,7 @@ __device__ __noinline__ bool task_panel_digits(unsigned char* sm, int kind, doub
     stg(Tg + (size_t)c0 * ib + o, Td[kb == 32 ? o : o % kb + o / kb * 32]);
   if (vd) {
     const double t[2] = {Td[arow + lane * 32], Td[arow + 1 + lane * 32]};
-    publish_t(vd, nb, t, true, nz, reinterpret_cast<uint32_t*>(colS));
+    publish_t(vd, nb, t, true, nz, strong, reinterpret_cast<uint32_t*>(colS));
     wait_image();
   }
   __syncthreads();

@@ -29,7 +29,8 @@
 // |V(r, j)| |W2(j, c)| < 2^-10 2^E_c for all j and c; or a pivot row j as small, under a reflector with next to no tail
 // (tau_j > 2 - 2^-14).  Rows of N(0, 1) columns have entries near 2^-4 2^E_c, so that full strips of ordinary matrices
 // never come to the second test (rows_lost).  In strips of fewer than 8 columns a row can be small by chance: there the
-// row of V has to be small too, |V(r, j)| < 2^-8 of the reflector's norm for all j.  Rows that no reflector touches are
+// row of V has to be small too, |V(r, j)| < 2^-8 ||v_j|| for all j (never with an entry of 2^-8, as ||v_j|| <= 1 beside the
+// unit entry).  Rows that no reflector touches are
 // not written back.
 //
 // Layout.  512 threads: thread t owns columns 16 (t / 256) .. + 15 of row t % 256 of the strip (int64 in registers;
@@ -245,7 +246,10 @@ __device__ __forceinline__ uint32_t abs_hi(int64_t x) {        // upper word of 
   const int h = (int)(x >> 32);
   return (uint32_t)(h ^ (h >> 31));
 }
+__device__ __forceinline__ uint32_t abs_hi(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
 constexpr uint32_t kSmallRow = 1u << (31 - 8);                 // 2^-8 of a column, in the upper word of C
+constexpr uint32_t kStrong = (1023u - 8) << 20;                // 2^-8, upper word in FP64 (compared as integers: FP64
+                                                               // comparisons take 16 cycles of the SM each)
 
 // Whether the block would lose a row's own scale (see the head of this file).  Thread: row r of the strip, 16 columns;
 // big: its largest |C| (abs_hi), nz: V has an entry in the row, w2: rows 2 warp, 2 warp + 1 of W2 2^(62 - E_c) in column
@@ -296,7 +300,8 @@ __device__ __noinline__ bool rows_lost(unsigned char* sm, int kb, int eT, uint32
 // Published blocks: what the updates of a reduction read of a panel block instead of V and T, made once by its factor
 // sub-task (a strip spent 4.4k of its 24k cycles a block on V's digits).  Digits of V in the operand layout
 // (digit_image_rows(nb) rows, zeros outside the block), T 2^(56 - eT) split as the updates read it, then the header: two
-// integers, whether |v| <= 1 and eT <= 12 hold, and eT, and from its word 4 on a bit for each row of V that is not zero.
+// integers, whether |v| <= 1 and eT <= 12 hold, and eT, from its word 4 on a bit for each row of V that is not zero and
+// from word 12 on for each with an entry of 2^-8 beside a unit one.
 // Starts the copy of the V area (16 KB a digit) into block vd; wait_image before the sub-task ends.
 __device__ __forceinline__ void store_image(unsigned char* sm, unsigned char* vd, int nb) {
   if ((int)uniform(threadIdx.x >> 5) == kIssueWarp) {
@@ -316,15 +321,17 @@ __device__ __forceinline__ void wait_image() {
   }
 }
 // T and the header; t: rows 2 warp, 2 warp + 1 of column lane, good: the block's V is in range (any thread), nz: this
-// thread's half of row r of V has an entry.
-__device__ __forceinline__ void publish_t(unsigned char* vd, int nb, const double* t, bool good, bool nz, uint32_t* red) {
+// thread's half of row r of V has an entry, strong: one of 2^-8; red: 48 words.
+__device__ __forceinline__ void publish_t(unsigned char* vd, int nb, const double* t, bool good, bool nz, bool strong,
+                                          uint32_t* red) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t h = max((uint32_t)__double2hiint(t[0]) & 0x7fffffffu, (uint32_t)__double2hiint(t[1]) & 0x7fffffffu);
   const uint32_t hm = __reduce_max_sync(kFull, h);
-  const unsigned rows = __ballot_sync(kFull, nz);
+  const unsigned rows = __ballot_sync(kFull, nz), big = __ballot_sync(kFull, strong);
   if (lane == 0) {
     red[warp] = hm;
     red[16 + warp] = rows;
+    red[32 + warp] = big;
   }
   const bool v_ok = __syncthreads_and(good ? 1 : 0) != 0;
   const int eT = max((int)(__reduce_max_sync(kFull, red[lane & 15]) >> 20) - 1022, 1);
@@ -337,15 +344,17 @@ __device__ __forceinline__ void publish_t(unsigned char* vd, int nb, const doubl
   }
   unsigned char* head = vd + digit_block_bytes(nb) - kDigitHeadBytes;
   if (threadIdx.x == 0) __stcg(reinterpret_cast<int2*>(head), make_int2(v_ok && eT <= 12 ? 1 : 0, eT));
-  if (threadIdx.x < 8)
-    __stcg(reinterpret_cast<uint32_t*>(head) + 4 + threadIdx.x, red[16 + threadIdx.x] | red[24 + threadIdx.x]);
+  if (threadIdx.x < 16) {
+    const int o = 16 + (threadIdx.x & 7) + 2 * (threadIdx.x & 8);
+    __stcg(reinterpret_cast<uint32_t*>(head) + 4 + threadIdx.x, red[o] | red[o + 8]);
+  }
 }
 // Publishes a block that task_panel_factor has just written.
 __device__ __noinline__ void publish_block(unsigned char* sm, int kind, const double* X, int tr, const double* Tg, int nb,
                                            int ib, int b, unsigned char* vd) {
   const int tid = threadIdx.x, kb = ib, c0 = b * ib, r = tid & 255, cb = 16 * (tid >> 8);
   const int r0 = kind == PM_GE ? c0 : 0, r1 = kind == PM_TT ? c0 + kb : nb;
-  bool good = true, nz = false;
+  bool good = true, nz = false, strong = false;
   __syncthreads();
 #pragma unroll
   for (int g = 0; g < 2; ++g) {
@@ -358,9 +367,10 @@ __device__ __noinline__ void publish_block(unsigned char* sm, int kind, const do
         if (kind == PM_TS || (kind == PM_GE ? d > 0 : d <= 0)) x = ldg(X + toff(r, c0 + c, nb, tr));
         if (kind == PM_GE && d == 0) x = 1.0;
       }
-      good = good && ((uint32_t)__double2hiint(x) & 0x7fffffffu) <= 0x3ff00000u;
-      if (((uint32_t)__double2hiint(x) & 0x7fffffffu) != 0)      // (not the unit entry of H = I)
-        nz = nz || kind != PM_GE || d != 0 || ldg(Tg + (size_t)c0 * ib + c * (kb + 1)) != 0.0;
+      good = good && abs_hi(x) <= 0x3ff00000u;
+      if (abs_hi(x) != 0)                // (not the unit entry of H = I)
+        nz = nz || kind != PM_GE || d != 0 || abs_hi(ldg(Tg + (size_t)c0 * ib + c * (kb + 1))) != 0;
+      strong = strong || (abs_hi(x) >= kStrong && !(kind == PM_GE && d == 0));
       v[a] = to_fixed(x, 62);
     }
     put_digits(sm + kDigV, r, (cb >> 3) + g, v);
@@ -372,7 +382,7 @@ __device__ __noinline__ void publish_block(unsigned char* sm, int kind, const do
   double t[2];
 #pragma unroll
   for (int k = 0; k < 2; ++k) t[k] = (arow + k < kb && lane < kb) ? ldg(Tg + (size_t)c0 * ib + arow + k + lane * kb) : 0.0;
-  publish_t(vd, nb, t, good, nz, reinterpret_cast<uint32_t*>(sm + kDigHead + 128));
+  publish_t(vd, nb, t, good, nz, strong, reinterpret_cast<uint32_t*>(sm + kDigHead + 128));
   wait_image();
   __syncthreads();
 }
@@ -531,7 +541,7 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
   const int myE = colE[lane];          // of column c = lane (the pivot rows' column)
   const uint32_t* rw = reinterpret_cast<const uint32_t*>(sm + kDigRow);
   const int ncols_nz = (int)(rw[16] + rw[17]);         // columns that are not zero
-  const bool small_row = ncols_nz > 0 && !row_bit(rw);
+  const bool small_row = ncols_nz > 0 && !row_bit(rw), narrow = ncols_nz < 8;
   bool touched = false;                // a reflector applied so far has an entry in row r
   bool ok = true;                      // this thread's completion waits
   for (int bb = 0; bb < nbk; ++bb) {
@@ -553,7 +563,7 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
     } else {
       ok = wait_v() && ok;
       if (tr) __syncthreads();
-      uint32_t hv = 0;                   // largest |v| (high word)
+      uint32_t hv = 0, hu = 0;           // largest |v| (high word), and beside the unit entries
       {
         const bool vrow = r >= v0 && r < v1;
 #pragma unroll
@@ -576,7 +586,10 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
           const int d = r - (c0 + cb + 8 * g);            // 0 on the diagonal of column a = 0
           if (type == UNMQR) {
 #pragma unroll
-            for (int a = 0; a < 8; ++a) x[a] = d > a ? x[a] : (d == a ? 1.0 : 0.0);
+            for (int a = 0; a < 8; ++a) {
+              hu = max(hu, in && d > a ? (uint32_t)__double2hiint(x[a]) & 0x7fffffffu : 0u);
+              x[a] = d > a ? x[a] : (d == a ? 1.0 : 0.0);
+            }
           } else if (type == TTMQR) {
 #pragma unroll
             for (int a = 0; a < 8; ++a) x[a] = d <= a ? x[a] : 0.0;
@@ -593,9 +606,11 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
         uint32_t ht = max((uint32_t)__double2hiint(tv[0]) & 0x7fffffffu, (uint32_t)__double2hiint(tv[1]) & 0x7fffffffu);
         ht = __reduce_max_sync(kFull, ht);
         const unsigned rows = __ballot_sync(kFull, hv != 0);
+        const unsigned big = __ballot_sync(kFull, (type == UNMQR ? hu : hv) >= kStrong);
         if (lane == 0) {
           red[warp] = ht;
           red[16 + warp] = rows;
+          red[32 + warp] = big;
         }
       }
       // the staged V is free from here on: the C digits take its place.  1: a wait ran out, 2: |v| > 1 (not finite)
@@ -719,10 +734,13 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
       for (int i = 0; i < 8; ++i) *reinterpret_cast<uint32_t*>(p + i * 2048) = d[i];
     }
     // ---- rows that fixed point would lose ------------------------------------------------------------
-    bool nz, pivot = false;            // V has an entry in row r; a pivot row is lost
+    bool nz, strong, pivot = false;    // V has an entry in row r, one of 2^-8; a pivot row is lost
     if constexpr (kPre) {
-      nz = (reinterpret_cast<const uint32_t*>(sm + kDigT + kDigTBytes)[4 + (warp & 7)] >> lane) & 1;
+      const uint32_t* hd = reinterpret_cast<const uint32_t*>(sm + kDigT + kDigTBytes) + 4 + (warp & 7);
+      nz = (hd[0] >> lane) & 1;
+      strong = (hd[8] >> lane) & 1;
     } else {
+      strong = row_bit(red + 32);
       nz = row_bit(red + 16);
       if (type == UNMQR && r >= c0 && r < c0 + kb && Ts[35 * (r - c0)].x == 0) {      // (not the unit entry of H = I)
         nz = false;
@@ -739,12 +757,12 @@ __device__ __noinline__ int task_update_digits(unsigned char* sm, int type, cons
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    if (__syncthreads_or(pivot || (small_row && nz))) {
+    if (__syncthreads_or(pivot || (small_row && nz && !(narrow && strong)))) {
       uint32_t big = 0;
 #pragma unroll
       for (int c = 0; c < 16; ++c) big = max(big, abs_hi(cf[c]));
       // uniform: the rest goes to the FP64 units
-      if (rows_lost(sm, kb, eT, big, nz, w2[0], w2[1], pivot, ncols_nz < 8, type == UNMQR ? c0 : -kDigRows)) {
+      if (rows_lost(sm, kb, eT, big, nz, w2[0], w2[1], pivot, narrow, type == UNMQR ? c0 : -kDigRows)) {
         if (!kPre && bb + 1 < nbk) ok = wait_v() && ok;
         break;
       }
