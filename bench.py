@@ -55,8 +55,8 @@ WORKLOADS = {
 # 2070 MHz = 1258.6 GFLOP/s.  Reported beside the measured peaks; the roofline of the adjoint divides by the
 # measured DFMA-loop rate (bidiag_measure_fp64_peaks), the FP64 unit its contractions run on.
 FP64_DERIVED_GFLOPS = 152 * 4 * 2.070
-# An FP64 reduction's contractions run as exact products of 8-bit digits on the f16 tensor pipe: seven digits an
-# operand, of whose pairs the 34 with i + j < 8 count (the rest weighs less than the rounding).
+# An FP64 reduction's contractions run as exact products of 8-bit digits on the f16 tensor pipe: of the pairs of seven
+# digits of V and of C the 34 with i + j < 8 (V W2, with eight digits of W2, has 35; the rate counts 34 for both).
 DIGIT_PRODUCTS = 34
 CPU_SAMPLE_SECONDS = 12.0
 
@@ -228,12 +228,15 @@ def trace_report(h, nb, ib, esize, nsm, title, w=32):
         s[2] += b
         s[3] += f or 0.0
     busy = dur.sum()
-    tc5 = int(((op >> 32) & 1).sum())
-    nupd = int(sum(1 for o in op if (int(o) & 15) in (1, 3, 5, 8)))
+    upd = np.isin(op & 15, (1, 3, 5, 8))
+    tc5, nupd = int(((op >> 32) & 1)[upd].sum()), int(upd.sum())
+    fac = (op & 15) == 7
+    tcf, nfac = int(((op >> 32) & 1)[fac].sum()), int(fac.sum())
     lines = [f"### {title}", "",
              f"launch span {1e-6 * (t1 - t0):.2f} ms, {n} sub-tasks, SMs busy {busy / (nsm * (t1 - t0)):.1%} "
              f"of the span ({nsm} SMs)" + (f"; {tc5} of {nupd} update sub-tasks ran C -= V W on tcgen05"
-                                           if tc5 else ""), "",
+                                           if tc5 else "")
+             + (f", {tcf} of {nfac} factors from Gram matrices" if tcf else ""), "",
              "| sub-task | count | total ms | share of busy | mean us | alg. bytes | GB/s | GFLOP/s |",
              "|---|---|---|---|---|---|---|---|"]
     for k in sorted(stats, key=lambda c: -stats[c][1]):

@@ -72,7 +72,7 @@ enum {
   BIDIAG_OPT_TIMING = 5,          /* 1: time the executor launch of each bidiag_band with CUDA events */
   BIDIAG_OPT_TRACE = 6,           /* 1: record a per-task trace of each bidiag_band (see bidiag_trace) */
   BIDIAG_OPT_F32_UPDATES = 7,     /* FP32 storage: 0 = updates as three TF32 tensor-core products, the
-                                     C -= V W product on tcgen05 (one matrix; default), 1 = updates by FP32
+                                     C -= V W product on tcgen05 (default), 1 = updates by FP32
                                      FMA on the CUDA cores (FP32-exact products), 2 = three TF32 products on
                                      the warp-level MMA only */
   BIDIAG_OPT_F32_SCALARS = 8,     /* FP32 storage: each reflector's beta, tau and tail scale from alpha and

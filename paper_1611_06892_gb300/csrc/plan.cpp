@@ -523,8 +523,9 @@ const AutotuneRow kAutotuneTable[] = {
 
 // Modelled time of a sub-task in units of 10 ns, dispatch (1 us) included (mode 1), from per-sub-task traces of
 // the executor on a GB300.  rows: rows of V; blocks: panel blocks an update strip applies.
-//  * FP64 digit products (nb 256, 192 and 128): factors and panel-block updates take the same time whatever the
-//    rows (their cost is per column), strips a fixed time per block.
+//  * FP64 digit products (measured at nb 256, 192 and 128, ib 32): factors and panel-block updates take the same time
+//    whatever the rows (their cost is per column), strips a fixed time per block.  Narrower inner blocks get the same
+//    factor times, though theirs are shorter (nb 64, ib 16: 41 - 57 us against 55 - 67).
 //  * FP32 storage with tcgen05 updates (ib 32, nb 256 and 128): factors and panel-block updates affine in the rows,
 //    strips in the flops.
 //  * Else the autotuner's table (strips of 32 columns) at the nearest tile size, in proportion to the flops (factors:
@@ -572,7 +573,7 @@ static int64_t sub_time(int64_t flops, int cls, int64_t rows, int nb, int ib, in
   return kDispatch + (int64_t)(100.0 * us);
 }
 
-// Queue order: the order in which a list schedule on the chip's SMs starts the sub-tasks (of the ready ones the one
+// Queue order: the order in which a list schedule on a GB300's 152 SMs starts the sub-tasks (of the ready ones the one
 // with the longest weighted path to the end first), by the modelled times.  CTAs take the queue strictly in order, so
 // a queue sorted by that path alone let them wait on sub-tasks of the chain while ready strips stood behind them
 // (GB300, that order against this one: 8192^2 FP64 181.1 -> 170.0 ms, FP32 96.3 -> 89.4, 4096^2 45.1 -> 42.4, a batch
